@@ -43,11 +43,11 @@ fr_status ensure_mt(fr_ctx *ctx, int n, int nnz, int k, int P) {
     }
     size_t b = 0;
     auto add = [&](size_t elem, long long cnt) { b += ((elem * (size_t)cnt + 255) / 256) * 256; };
-    add(4, nn); add(8, nn); add(4, 1); add(1, nn);      // tch cur epoch mvd
-    add(16, nn); add(4, nn);                            // lmv kept
+    add(64, nn);                                        // rec (four int4 per vertex)
+    add(8, nn); add(4, nn);                             // lmv kept
     const long long kwch = (nn + kKwChunk - 1) / kKwChunk + 1;
-    add(4, (2 * kwch + 1) * kMtBuckets);                // kwtab
-    add(32, ecap);                                      // ent (two int4 per entry)
+    add(4, (kwch + 1) * kMtBuckets);                // kwtab
+    add(16, ecap);                                      // ent
     add(4, kk);                                         // bpair
     add(4, pp); add(4, pp); add(4, pp); add(4, pp);     // pa pb cnt fil
     add(8, pp + 1);                                     // off
@@ -69,12 +69,11 @@ fr_status ensure_mt(fr_ctx *ctx, int n, int nnz, int k, int P) {
     ctx->mt_n = (int)nn; ctx->mt_nnz = (int)mm; ctx->mt_k = kk; ctx->mt_p = pp;
     char *p = reinterpret_cast<char *>(ctx->mt_mem);
     MtDev &m = ctx->mt;
-    m.tch = carve_mt<int>(p, nn); m.cur = carve_mt<unsigned long long>(p, nn); m.epoch = carve_mt<unsigned>(p, 1);
-    m.mvd = carve_mt<unsigned char>(p, nn);
-    m.lmv = carve_mt<int4>(p, nn); m.kept = carve_mt<int>(p, nn);
-    m.kwtab = carve_mt<int>(p, (2 * kwch + 1) * kMtBuckets);
+    m.rec = carve_mt<int4>(p, 4 * nn);
+    m.lmv = carve_mt<int2>(p, nn); m.kept = carve_mt<int>(p, nn);
+    m.kwtab = carve_mt<int>(p, (kwch + 1) * kMtBuckets);
     m.kwchunks = (int)kwch;
-    m.ent = carve_mt<int4>(p, 2 * ecap);
+    m.ent = carve_mt<int4>(p, ecap);
     m.bpair = carve_mt<int>(p, kk);
     m.pa = carve_mt<int>(p, pp); m.pb = carve_mt<int>(p, pp); m.cnt = carve_mt<int>(p, pp); m.fil = carve_mt<int>(p, pp);
     m.off = carve_mt<long long>(p, pp + 1);
@@ -82,10 +81,6 @@ fr_status ensure_mt(fr_ctx *ctx, int n, int nnz, int k, int P) {
     m.bw = carve_mt<long long>(p, kk); m.chg = carve_mt<unsigned char>(p, kk);
     m.res = carve_mt<MtRes>(p, 1);
     m.ecap = ecap; m.scap = scap;
-    // versions start at zero; the moved marks are zero between searches
-    CK(cudaMemsetAsync(m.cur, 0, sizeof(unsigned long long) * (size_t)nn, ctx->stream));
-    CK(cudaMemsetAsync(m.epoch, 0, sizeof(unsigned), ctx->stream));
-    CK(cudaMemsetAsync(m.mvd, 0, (size_t)nn, ctx->stream));
     return FR_OK;
 }
 

@@ -11,6 +11,8 @@ namespace fr {
 constexpr int kMtGmax = 1023;                 // |gain| bound (max weighted degree)
 constexpr int kMtBuckets = 2 * kMtGmax + 2;   // gain buckets of the single queue
 constexpr int kMtMaxK = 1024;                 // block weights cached in shared memory
+constexpr int kMtRing = 2048;                 // latest entries of a search kept in shared memory (a power of two)
+constexpr int kMtLast = 256;                  // last moves of a search kept there (a power of two)
 constexpr int kKwChunk = 1024;                // start entries per warp when a round's queue is built
 
 // Totals of one pass.
@@ -20,22 +22,18 @@ struct MtRes {
     int stopped;             // global k-way round: 1 if the KaSPar rule stopped its search
 };
 
-// Device state of a multi-try pass over the pairs of one matching of one graph.
-// Per-vertex arrays: tch is cleared before every pass (by the launcher); mvd is zero
-// between searches; cur is meaningful only for the current search's epoch.
+// Device state of a multi-try pass over the pairs of one matching of one graph.  The
+// records are built before every pass and every global round.
 struct MtDev {
-    int *tch;                    // [n] search of this pass that queued the vertex, 0 = none
-    unsigned long long *cur;     // [n] epoch << 32 | the vertex's latest entry in that search
-    unsigned *epoch;             // [1] epoch of the last search run (searches number 1, 2, ...)
-    unsigned char *mvd;          // [n] moved by the current search
-    int4 *lmv;                   // [n] moves of the current search: {vertex, source, target, weight}
+    int4 *rec;                   // [4 n] vertex records: row, block, marks, connection weights
+    int2 *lmv;                   // [n] moves of the current search: {vertex, source << 10 | target}
     int *kept;                   // [n] the pass's kept movers (a vertex moves at most once in a pass)
     int *kwtab;                  // global rounds: per chunk of the start set and gain bucket, the
-                                 // chunk's last entry, then the last entry before the chunk
-                                 // (2 x kwchunks x kMtBuckets), then each bucket's top (kMtBuckets)
+                                 // chunk's entries, then the bucket's entries before the chunk
+                                 // (kwchunks x kMtBuckets), then each bucket's entries (kMtBuckets)
     int kwchunks;                // chunks the table holds (ceil(n / kKwChunk) + 1)
-    int4 *ent;                   // [2 ecap] bucket stack entries of the current search:
-                                 //   {vertex, entry below, live, target}, {block, weight, adjacency range}
+    int4 *ent;                   // [ecap] bucket stack entries of the current search:
+                                 //   {vertex, entry below, live | degree | block | target, row begin}
     int *bpair;                  // [k] pair of the pass that the block belongs to, -1 none
     int *pa, *pb;                // [P] the pairs, in pass order
     int *cnt, *fil;              // [P] todo list lengths, fill cursors
