@@ -41,7 +41,9 @@ QCaps caps_for(int ctas, int n) {
     c.nu = (long long)ctas * dyn / 28 + 64;
     c.mu = (long long)ctas * dyn / 16 + 64;
     c.vq = std::min<long long>(n, std::max<long long>(4 * c.nu, 1 << 16));
-    c.words = n / 32 + 2;
+    // the ids are numbered a group of 1,024 at a time, so the last group's words are read to
+    // its end: they exist, and are cleared with the others
+    c.words = 32LL * (n / 1024 + 1);
     c.swords = n / 32768 + 2;
     return c;
 }
