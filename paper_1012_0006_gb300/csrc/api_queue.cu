@@ -34,7 +34,9 @@ struct QCaps {
 };
 
 // Per-pair capacities of a cluster of `ctas` CTAs: a network that fits its shared
-// memory has at most dyn / 29 vertices and dyn / 16 arcs per CTA.
+// memory has at most dyn / 29 vertices; arcs have room for dyn / 16 per CTA (8 bytes each
+// would fit, but a pair that large is better off on a larger cluster, and the HBM arrays of
+// every slot would double).
 QCaps caps_for(int ctas, int n) {
     const long long dyn = (long long)queue_smem();
     QCaps c;
@@ -198,7 +200,8 @@ int queue_size_for(fr_ctx *ctx, const BatchPlan &pl, const fr_options *opt) {
     if (dyn == 0) return -1;
     long long est = 0;
     for (long long e : pl.est_max) est = std::max(est, e);
-    const double need = 1.05 * (double)est * (29.0 + (ctx->narrow_ok ? 16.0 : 20.0) * pl.avg_degree);
+    // (16 bytes an arc: the arcs a slot has room for, see caps_for)
+    const double need = 1.05 * (double)est * (29.0 + 16.0 * pl.avg_degree);
     const double per_cta = 0.95 * (double)dyn;
     const int force = opt->cluster_ctas ? opt->cluster_ctas : ctx->tune_ctas;
     int best = -1;

@@ -33,11 +33,16 @@ struct ClusterHdr {
     int kloc[3][kClusterMax + 1];   // candidate splits (by arcs, by bytes, by vertices; CTA 0's copy)
     int cabc[3][kClusterMax + 1];
     int grab[2];                // slot of the size order taken (CTA 0's copy, by parity)
+    int nrem;                   // remote arcs of this CTA
+    int qn[3];                  // entries of the outgoing queue, rotating
+    int wn[2];                  // entries of the worklist, by parity
+    int any[3];                 // rotating votes (each CTA's copy holds the cluster's)
     long long flow;
 };
+static_assert(sizeof(ClusterHdr) <= kHdrBytes, "the header leads the dynamic shared memory");
 
 // Distributed shared memory by explicit address: a shared::cluster address (32 bits) of an
-// element of some CTA's shared memory, and plain stores / relaxed reductions to it.  Every
+// element of some CTA's shared memory, and plain loads / relaxed reductions at it.  Every
 // CTA carves its arrays at the same offsets, so the address of array X at the same index
 // is the address of array Y plus a fixed byte offset.
 __device__ __forceinline__ unsigned cta_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -45,6 +50,11 @@ __device__ __forceinline__ unsigned map_rank(unsigned a, int rank) {
     unsigned r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
     return r;
+}
+__device__ __forceinline__ int dsm_ld(unsigned a) {
+    int v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
 }
 __device__ __forceinline__ void dsm_st(unsigned a, int v) {
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
@@ -62,6 +72,23 @@ __device__ __forceinline__ void dsm_or(unsigned a, int v) {
     asm volatile("red.shared::cluster.or.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 
+// An array in the dynamic shared memory, by its byte offset there: the compiler sees that
+// every access is to shared memory (through a pointer kept in a struct it may not).
+template <class T>
+struct ShArr {
+    unsigned o;
+    __device__ __forceinline__ T *ptr() const {
+        extern __shared__ __align__(16) char csmem[];
+        return reinterpret_cast<T *>(csmem + o);
+    }
+    __device__ __forceinline__ T &operator[](int i) const { return ptr()[i]; }
+};
+
+template <int N>
+struct Int {
+    __device__ constexpr int operator()() const { return N; }
+};
+
 template <int TPB>
 struct ClusterFlow {
     const Work &w;
@@ -69,8 +96,12 @@ struct ClusterFlow {
     const int rank, C;
     ClusterHdr *hdr;
     ClusterHdr *hdr0;          // CTA 0's header
+    static __device__ __forceinline__ ClusterHdr *H() {   // this CTA's
+        extern __shared__ __align__(16) char csmem[];
+        return reinterpret_cast<ClusterHdr *>(csmem);
+    }
     // local arrays
-    int *lab, *ex, *fx, *cofs, *gidx, *rfl, *cla, *res, *csum;
+    ShArr<int> lab, ex, fx, cofs, gidx, rfl, cla, res, csum;
     // narrow: every capacity sum csum(a) = c(a) + c(reverse a) is below 2^16, and
     // res[a] holds res(a) | csum(a) << 16 (csum unused); additions to the residual
     // never carry into the upper half because res(a) <= csum(a)
@@ -81,67 +112,147 @@ struct ClusterFlow {
     }
     __device__ __forceinline__ int cs(int a) const { return narrow ? (int)((unsigned)res[a] >> 16) : csum[a]; }
     __device__ __forceinline__ void set_rs(int a, int v) { res[a] = narrow ? ((res[a] & ~0xFFFF) | v) : v; }
-    // per arc: shared::cluster addresses of the head's label (hadr) and of the reverse
-    // arc's residual (radr); other arrays of the same element are a fixed offset away
-    unsigned *hadr, *radr;
-    unsigned o_ex, o_rfl, o_cla, o_hlab;   // byte offsets: ex/rfl/cla from lab, hlab from res
-    int *hlab;                 // per arc: the label of its head as last published by the head
-    unsigned char *bord;
-    int rot;                   // rotating counter index (identical in every CTA)
+    // Per arc, one word.  An arc whose head this CTA holds: its rank, the head's index and
+    // the index of the reverse arc (a CTA's shared memory holds fewer than 2^13 vertices of
+    // 31 bytes and 2^15 arcs of 8).  An arc into another CTA: another rank, and a slot of the
+    // remote tables, which hold the same three for it (rw), a copy of the head's label (rg)
+    // and the slot of the reverse arc in the head's CTA (rslot).  With the residual an arc is
+    // 8 bytes, 18 if remote: cluster-wide addresses of both and a copy of every head's label
+    // took 16, and the widest pair of a 65,536-vertex 2D rgg (31,456 vertices, 248 K arcs)
+    // then fitted no cluster.
+    ShArr<unsigned> adr, rw;
+    ShArr<int> rg;
+    ShArr<unsigned short> rslot;
+    ShArr<unsigned short> wl;  // worklist: the vertices a pass or scan works on
+    unsigned lab0, res0, rg0, adr0;   // shared::cta addresses of lab, res, rg, adr
+    unsigned o_ex, o_rfl, o_cla;      // byte offsets: ex/rfl/cla from lab
+    ShArr<unsigned char> bord;
+    int rot, arot;             // rotating counter and vote indexes (identical in every CTA)
+
+    static constexpr int kVtxBits = 13, kArcBits = 15;
+    static __device__ __forceinline__ unsigned pack_adr(int rk, int v, int a) {
+        return ((unsigned)rk << (kVtxBits + kArcBits)) | ((unsigned)v << kArcBits) | (unsigned)a;
+    }
+    static __device__ __forceinline__ int adr_rank(unsigned w) { return (int)(w >> (kVtxBits + kArcBits)); }
+    static __device__ __forceinline__ int adr_vtx(unsigned w) { return (int)(w >> kArcBits) & ((1 << kVtxBits) - 1); }
+    static __device__ __forceinline__ int adr_arc(unsigned w) { return (int)(w & ((1u << kArcBits) - 1)); }
+    static __device__ __forceinline__ int adr_slot(unsigned w) { return (int)(w & ((1u << (kVtxBits + kArcBits)) - 1)); }
+    __device__ __forceinline__ bool local(unsigned w) const { return adr_rank(w) == rank; }
+    // of a remote table word: the head in the array `off` bytes after lab, the reverse
+    // arc's residual
+    __device__ __forceinline__ unsigned head_at(unsigned w, unsigned off = 0) const {
+        return map_rank(lab0 + off + 4 * adr_vtx(w), adr_rank(w));
+    }
+    __device__ __forceinline__ unsigned rev_at(unsigned w) const {
+        return map_rank(res0 + 4 * adr_arc(w), adr_rank(w));
+    }
+    // label of an arc's head: exact in this CTA, the copy elsewhere
+    __device__ __forceinline__ int head_label(unsigned w) const {
+        return *(volatile int *)(local(w) ? &lab[adr_vtx(w)] : &rg[adr_slot(w)]);
+    }
+
+    // Updates of other CTAs' memory go through a queue in shared memory, sent 32 entries an
+    // instruction after a block barrier: an instruction that reaches another CTA holds its
+    // warp 200-370 cycles, however few lanes take part.  Sent arc by arc as they arise (one
+    // in seven, in nearly every instruction) they made up most of the flow's time.  Two
+    // halves and three counters rotate, so a barrier before the sending is all it needs; an
+    // entry that finds its half full is sent at once.
+    enum { Q_PUSH = 0, Q_LABEL = 1, Q_MIN = 2, Q_OR = 3, Q_MAX = 4 };
+    static constexpr int kQueue = 512;   // entries of a half
+    ShArr<int2> queue;
+    int qrot;                            // block barriers passed by the queue (the same in every thread)
+
+    __device__ __forceinline__ void send(int op, int slot, int val) const {
+        const unsigned w = rw[slot];
+        if (op == Q_PUSH) {
+            dsm_add(rev_at(w), val);
+            dsm_add(head_at(w, o_ex), val);
+        } else if (op == Q_LABEL) {
+            dsm_st(map_rank(rg0 + 4 * rslot[slot], adr_rank(w)), val);
+        } else if (op == Q_MIN) {
+            dsm_min(head_at(w), val);
+        } else if (op == Q_OR) {
+            dsm_or(head_at(w, o_rfl), val);
+        } else {
+            dsm_max(head_at(w, o_cla), val);
+        }
+    }
+    __device__ __forceinline__ void enqueue(int op, int slot, int val) {
+        const int at = atomicAdd(&H()->qn[qrot % 3], 1);
+        if (at < kQueue) queue[(qrot & 1) * kQueue + at] = make_int2(op << 28 | slot, val);
+        else send(op, slot, val);
+    }
+    // Every thread of the CTA: ends a pass or scan, with a block barrier, and sends.
+    __device__ __forceinline__ void flush() {
+        if (threadIdx.x == 0) H()->qn[(qrot + 1) % 3] = 0;   // (last read before the previous barrier)
+        __syncthreads();
+        const int n = min(*(volatile int *)&H()->qn[qrot % 3], kQueue);
+        for (int i = threadIdx.x; i < n; i += TPB) {
+            const int2 q = queue[(qrot & 1) * kQueue + i];
+            send((int)((unsigned)q.x >> 28), q.x & 0xfffffff, q.y);
+        }
+        ++qrot;
+    }
+
+    // The vertices of this CTA that pred holds for go on the worklist (one reservation per
+    // warp); returns their number, the same in every thread, behind a block barrier.  The
+    // work on them is then shared evenly over the warps (each): the vertices with
+    // something to do lie together, and the warp that holds most of them made a pass over the
+    // CTA's own strips last several times the average.
+    int wrot;
+    template <class Pred>
+    __device__ __forceinline__ int collect(int nv, Pred pred) {
+        const int lane = threadIdx.x & 31;
+        int *wn = &H()->wn[wrot & 1];
+        for (int base = threadIdx.x - lane; base < nv; base += TPB) {
+            const int lv = base + lane;
+            const bool f = lv < nv && pred(lv);
+            const unsigned m = __ballot_sync(FULL, f);
+            if (!m) continue;
+            int at = 0;
+            if (lane == 0) at = atomicAdd(wn, __popc(m));
+            at = __shfl_sync(FULL, at, 0);
+            if (f) wl[at + __popc(m & ((1u << lane) - 1u))] = (unsigned short)lv;
+        }
+        __syncthreads();
+        const int n = *(volatile int *)wn;
+        ++wrot;
+        if (threadIdx.x == 0) H()->wn[wrot & 1] = 0;   // (last read before the previous flush's barrier)
+        return n;
+    }
+    // f(u, gl) for every vertex u of the worklist (n of them), G lanes each (gl of G); on
+    // all lanes of a warp together, u = -1 where a group has none.
+    template <int G, class Fn>
+    __device__ __forceinline__ void each(int n, Fn f) {
+        const int lane = threadIdx.x & 31;
+        for (int b = (int)(threadIdx.x >> 5) * (32 / G); b < n; b += TPB / G) {
+            const int i = b + lane / G;
+            f(i < n ? (int)wl[i] : -1, lane % G);
+        }
+    }
 
     static constexpr int U = 8;   // arcs whose loads are issued together
 
-    // Lowest head label over the residual arcs [a0, a1) (res > 0), and the arc holding
-    // it.  Reads only this CTA's memory: the arcs' copies of their head labels.
-    __device__ __forceinline__ void lowest(int a0, int a1, int &hmin, int &best) const {
-        hmin = INT_MAX;
-        best = -1;
-        for (int a = a0; a < a1; a += U) {
-            int r[U], l[U];
+    // Calls f(word, res, csum) for arcs gl, gl + G, ... of vertex u's row, four at a time with
+    // their loads issued together (one arc after the other is a chain of shared
+    // memory loads and branches: a relabel of a 3D rgg pair took 80 K cycles so).
+    template <int G, class Fn>
+    __device__ __forceinline__ void walk(int u, int gl, Fn f) const {
+        const int a1 = cofs[u + 1];
+        for (int a = cofs[u] + gl; a < a1; a += 4 * G) {
+            unsigned w4[4];
+            int r[4], c[4];
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                r[u] = a + u < a1 ? rs(a + u) : 0;
-                l[u] = a + u < a1 ? *(volatile int *)&hlab[a + u] : INT_MAX;
+            for (int i = 0; i < 4; ++i) {
+                const int x = a + i * G;
+                w4[i] = x < a1 ? adr[x] : 0u;
+                const int v = x < a1 ? *(volatile int *)&res[x] : 0;
+                r[i] = narrow ? v & 0xFFFF : v;
+                c[i] = narrow ? (int)((unsigned)v >> 16) : x < a1 ? csum[x] : 0;
             }
 #pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (r[u] > 0 && l[u] < hmin) { hmin = l[u]; best = a + u; }
+            for (int i = 0; i < 4; ++i) f(w4[i], r[i], c[i]);   // (past the row: res = csum = 0)
         }
-    }
-
-
-    // Runs f(src, gl, G) once on every lane for the flagged vertices among this
-    // warp's 32 (flag is the lane's own vertex, base + lane).  Up to eight flagged:
-    // group g = lane / 4 takes the g-th of them, src = its lane (-1: none for this
-    // group), gl = lane % 4 the lane's place in the group, G = 4, so a vertex's arcs
-    // are walked four at a time.  More than eight: each lane takes its own vertex
-    // (src = lane or -1, gl = 0, G = 1).  f gets per-vertex values from lane src with
-    // __shfl_sync on all lanes before it tests src.
-    template <class Fn>
-    __device__ __forceinline__ void for_flagged(bool flag, Fn f) const {
-        const int lane = threadIdx.x & 31;
-        const unsigned m = __ballot_sync(FULL, flag);
-        if (!m) return;
-        if (__popc(m) > 8) {
-            f(flag ? lane : -1, 0, 1);
-            return;
-        }
-        unsigned mm = m;
-        for (int i = 0; i < (lane >> 2); ++i) mm &= mm - 1;
-        f(mm ? __ffs(mm) - 1 : -1, lane & 3, 4);
-    }
-
-    // New label h of local vertex lv: its own word and the copies on the reverse
-    // arcs of its arcs (the arcs of which lv is the head), local or in other CTAs.
-    // The copies may lag; they never run ahead of the label, and labels only rise
-    // between exact relabels, so a lagging copy only makes a push look admissible
-    // that is not -- capacities and excesses stay exact, and a phase ends only once
-    // exact labels (phase 1) or the residual sets (phase 0) show that no excess can
-    // still reach its target.
-    __device__ __forceinline__ void set_label(int lv, int h) {
-        lab[lv] = h;
-        const int a1 = cofs[lv + 1];
-        for (int a = cofs[lv]; a < a1; ++a) dsm_st(radr[a] + o_hlab, h);
     }
 
     __device__ ClusterFlow(const Work &w_, char *smem)
@@ -149,7 +260,8 @@ struct ClusterFlow {
           C((int)cg::this_cluster().num_blocks()) {
         hdr = reinterpret_cast<ClusterHdr *>(smem);
         hdr0 = cl.map_shared_rank(hdr, 0);
-        rot = 0;
+        rot = arot = 0;
+        qrot = wrot = 0;
     }
 
     long long nsync = 0;       // cluster barriers of the current pair (CTA 0, thread 0)
@@ -157,6 +269,19 @@ struct ClusterFlow {
     __device__ void sync() {
         ++nsync;
         cl.sync();
+    }
+
+    // True if x holds for any thread of the cluster: a block vote, then one instruction sets
+    // every CTA's copy, so that after the one cluster barrier each reads its own.  (A copy's
+    // next slot was last read before the previous barrier, so its CTA may clear it now.)
+    __device__ bool cluster_any(bool x) {
+        const int s = __syncthreads_or(x);
+        if (s && threadIdx.x < C) dsm_or(map_rank(cta_addr(&H()->any[arot]), (int)threadIdx.x), 1);
+        if (threadIdx.x == 0) H()->any[(arot + 1) % 3] = 0;
+        sync();
+        const bool r = *(volatile int *)&H()->any[arot] != 0;
+        arot = (arot + 1) % 3;
+        return r;
     }
 
     // Cluster-wide sum of x (one value per thread); every thread gets the total.
@@ -173,48 +298,58 @@ struct ClusterFlow {
         if ((threadIdx.x & 31) == 0 && x) {
             if (is_max) atomicMax(c, x); else atomicAdd(c, x);
         }
-        if (rank == 0 && threadIdx.x == 0) hdr->cnt[(rot + 1) % 3] = 0;
+        if (rank == 0 && threadIdx.x == 0) H()->cnt[(rot + 1) % 3] = 0;
         sync();
         const int tot = *(volatile int *)c;
         rot = (rot + 1) % 3;
         return tot;
     }
 
-    __device__ void carve(char *smem, int nvcap, int nacap, bool narrow_) {
+    int nrcap;                 // remote arcs the tables have room for (the same in every CTA)
+    __device__ void carve(size_t smem_bytes, int nvcap, int nacap, bool narrow_) {
         narrow = narrow_;
-        char *p = smem + kHdrBytes;
-        auto take = [&](size_t bytes) {
-            char *r = p;
+        unsigned p = kHdrBytes;
+        auto take = [&](unsigned bytes) {
+            const unsigned r = p;
             p += (bytes + 15) / 16 * 16;
             return r;
         };
-        lab = reinterpret_cast<int *>(take(4ull * nvcap));
-        ex = reinterpret_cast<int *>(take(4ull * nvcap));
-        fx = reinterpret_cast<int *>(take(4ull * nvcap));
-        cofs = reinterpret_cast<int *>(take(4ull * (nvcap + 1)));
-        gidx = reinterpret_cast<int *>(take(4ull * nvcap));
-        rfl = reinterpret_cast<int *>(take(4ull * nvcap));
-        cla = reinterpret_cast<int *>(take(4ull * nvcap));
-        bord = reinterpret_cast<unsigned char *>(take(nvcap));
-        hadr = reinterpret_cast<unsigned *>(take(4ull * nacap));
-        radr = reinterpret_cast<unsigned *>(take(4ull * nacap));
-        res = reinterpret_cast<int *>(take(4ull * nacap));
-        csum = narrow ? nullptr : reinterpret_cast<int *>(take(4ull * nacap));
-        hlab = reinterpret_cast<int *>(take(4ull * nacap));
-        o_ex = cta_addr(ex) - cta_addr(lab);
-        o_rfl = cta_addr(rfl) - cta_addr(lab);
-        o_cla = cta_addr(cla) - cta_addr(lab);
-        o_hlab = cta_addr(hlab) - cta_addr(res);
+        lab.o = take(4u * nvcap);
+        ex.o = take(4u * nvcap);
+        fx.o = take(4u * nvcap);
+        cofs.o = take(4u * (nvcap + 1));
+        gidx.o = take(4u * nvcap);
+        rfl.o = take(4u * nvcap);
+        cla.o = take(4u * nvcap);
+        bord.o = take(nvcap);
+        wl.o = take(2u * nvcap);
+        adr.o = take(4u * nacap);
+        res.o = take(4u * nacap);
+        csum.o = narrow ? 0u : take(4u * nacap);
+        queue.o = take(2 * kQueue * sizeof(int2));
+        // the rest: the remote tables
+        nrcap = (int)(smem_bytes - p - 48) / 10;
+        rw.o = take(4u * nrcap);
+        rg.o = take(4u * nrcap);
+        rslot.o = p;
+        lab0 = cta_addr(lab.ptr());
+        res0 = cta_addr(res.ptr());
+        rg0 = cta_addr(rg.ptr());
+        adr0 = cta_addr(adr.ptr());
+        o_ex = ex.o - lab.o;
+        o_rfl = rfl.o - lab.o;
+        o_cla = cla.o - lab.o;
     }
 
     static __host__ __device__ size_t bytes_for(int nvcap, int nacap, bool narrow) {
         auto a = [](size_t b) { return (b + 15) / 16 * 16; };
-        return kHdrBytes + 7 * a(4ull * nvcap) + a(4ull * (nvcap + 1)) + a(nvcap) + (narrow ? 4 : 5) * a(4ull * nacap);
+        return kHdrBytes + 7 * a(4ull * nvcap) + a(4ull * (nvcap + 1)) + a(nvcap) + a(2ull * nvcap) + (narrow ? 2 : 3) * a(4ull * nacap) +
+               2 * kQueue * sizeof(int2) + 64;
     }
 
     __device__ int owner(int k) const {   // CTA whose range holds member k
         int r = 0;
-        while (r + 1 < C && hdr->klo[r + 1] <= k) ++r;
+        while (r + 1 < C && H()->klo[r + 1] <= k) ++r;
         return r;
     }
 
@@ -276,14 +411,14 @@ struct ClusterFlow {
         sync();
         // arc and shared-memory byte prefixes over members (each CTA a slice of the
         // member list, each thread a contiguous part of it), and three candidate splits
-        // into C contiguous ranges: equal arcs (the work of the flow), equal bytes (29
-        // per vertex, 16 or 20 per arc) and equal vertices.  Every CTA carves its arrays
+        // into C contiguous ranges: equal arcs (the work of the flow), equal bytes (31
+        // per vertex, 8 or 12 per arc) and equal vertices.  Every CTA carves its arrays
         // for the largest range's vertices and arcs, so the first candidate that fits
         // shared memory is taken: the arc split where it fits, the others where the
         // order of the vertices puts many light vertices together.
-        const int ab = w.narrow ? 16 : 20;
+        const int ab = w.narrow ? 8 : 12;
         {
-            const long long Btot = 29LL * V + (long long)ab * A;
+            const long long Btot = 31LL * V + (long long)ab * A;
             const long long tot3[3] = {(long long)A, Btot, (long long)V};
             const int per = (V + C - 1) / C;
             const int k0 = min(V, per * rank), k1 = min(V, k0 + per);
@@ -296,7 +431,7 @@ struct ClusterFlow {
             }
             int tot, btot;
             const int e0 = block_exclusive_scan<TPB>(mine, &tot);
-            const int b0 = block_exclusive_scan<TPB>(29 * (s1 - s0) + ab * mine, &btot);
+            const int b0 = block_exclusive_scan<TPB>(31 * (s1 - s0) + ab * mine, &btot);
             if (threadIdx.x == 0) {
                 hdr0->counts[rank] = tot;
                 hdr0->counts2[rank] = btot;
@@ -315,18 +450,18 @@ struct ClusterFlow {
             // the range's first arc into CTA 0
             if (rank == 0 && threadIdx.x == 0) {
                 for (int c = 0; c < 3; ++c) {
-                    hdr->kloc[c][0] = 0;
-                    hdr->cabc[c][0] = 0;
-                    hdr->kloc[c][C] = V;
-                    hdr->cabc[c][C] = A;
+                    H()->kloc[c][0] = 0;
+                    H()->cabc[c][0] = 0;
+                    H()->kloc[c][C] = V;
+                    H()->cabc[c][C] = A;
                     for (int r = 1; r < C; ++r)
-                        if (tot3[c] * r / C <= 0) { hdr->kloc[c][r] = 0; hdr->cabc[c][r] = 0; }
+                        if (tot3[c] * r / C <= 0) { H()->kloc[c][r] = 0; H()->cabc[c][r] = 0; }
                 }
             }
             for (int k = s0; k < s1; ++k) {
                 const int i = __ldcg(&pmem[k]);
                 const int d = w.off[i + 1] - w.off[i];
-                const int b = 29 + ab * d;
+                const int b = 31 + ab * d;
                 pacs[k] = run;
                 const long long lo3[3] = {(long long)run, brun, (long long)k};
                 const long long sz3[3] = {(long long)d, (long long)b, 1};
@@ -349,45 +484,52 @@ struct ClusterFlow {
             for (int c = 0; c < 3; ++c) {
                 int nvc = 0, nac = 0;
                 for (int r = 0; r < C; ++r) {
-                    nvc = max(nvc, hdr->kloc[c][r + 1] - hdr->kloc[c][r]);
-                    nac = max(nac, hdr->cabc[c][r + 1] - hdr->cabc[c][r]);
+                    nvc = max(nvc, H()->kloc[c][r + 1] - H()->kloc[c][r]);
+                    nac = max(nac, H()->cabc[c][r + 1] - H()->cabc[c][r]);
                 }
                 pick = c;
                 if (bytes_for(nvc, nac, w.narrow != 0) <= smem_bytes) break;
             }
             for (int r = 0; r <= C; ++r) {
-                hdr->klo[r] = hdr->kloc[pick][r];
-                hdr->cab[r] = hdr->cabc[pick][r];
+                H()->klo[r] = H()->kloc[pick][r];
+                H()->cab[r] = H()->cabc[pick][r];
             }
         }
         sync();
         // the C ranges, copied from CTA 0 (same in every CTA)
         if (threadIdx.x <= C && rank != 0) {
-            hdr->klo[threadIdx.x] = *(volatile int *)&hdr0->klo[threadIdx.x];
-            hdr->cab[threadIdx.x] = *(volatile int *)&hdr0->cab[threadIdx.x];
+            H()->klo[threadIdx.x] = *(volatile int *)&hdr0->klo[threadIdx.x];
+            H()->cab[threadIdx.x] = *(volatile int *)&hdr0->cab[threadIdx.x];
         }
         __syncthreads();
         if (threadIdx.x == 0) {
             int nvcap = 0, nacap = 0;
             for (int r = 0; r < C; ++r) {
-                nvcap = max(nvcap, hdr->klo[r + 1] - hdr->klo[r]);
-                nacap = max(nacap, hdr->cab[r + 1] - hdr->cab[r]);
+                nvcap = max(nvcap, H()->klo[r + 1] - H()->klo[r]);
+                nacap = max(nacap, H()->cab[r + 1] - H()->cab[r]);
             }
-            hdr->nvcap = nvcap;
-            hdr->nacap = nacap;
+            H()->nvcap = nvcap;
+            H()->nacap = nacap;
         }
         __syncthreads();
-        const int nvcap = hdr->nvcap, nacap = hdr->nacap;
+        const int nvcap = H()->nvcap, nacap = H()->nacap;
         const bool nar = w.narrow != 0;
         unsigned long long t1 = t_in;
         mark(t1, T_CL_MEMBERS);
         if (bytes_for(nvcap, nacap, nar) > smem_bytes) return false;   // same decision in every CTA
-        carve(smem, nvcap, nacap, nar);
-        const int klo = hdr->klo[rank], khi = hdr->klo[rank + 1];
+        carve(smem_bytes, nvcap, nacap, nar);
+        if (threadIdx.x == 0) {
+            H()->nrem = 0;
+            H()->qn[0] = H()->qn[1] = H()->qn[2] = 0;
+            H()->any[0] = H()->any[1] = H()->any[2] = 0;
+            H()->wn[0] = H()->wn[1] = 0;
+        }
+        qrot = wrot = 0;
+        __syncthreads();
+        const int klo = H()->klo[rank], khi = H()->klo[rank + 1];
         const int nv = khi - klo;
-        const int abase = hdr->cab[rank];
+        const int abase = H()->cab[rank];
         // load this CTA's vertices and arcs
-        int nremote = 0;   // arcs whose head another CTA holds
         for (int lv = threadIdx.x; lv < nv; lv += TPB) {
             const int i = __ldcg(&pmem[klo + lv]);
             gidx[lv] = i;
@@ -422,10 +564,14 @@ struct ClusterFlow {
                     if (jb + u >= j1) break;
                     const int la = a0 + (jb + u - j0);
                     const int rh = owner(kh[u]);
-                    nremote += rh != rank;
-                    hadr[la] = map_rank(cta_addr(lab + (kh[u] - hdr->klo[rh])), rh);
-                    const int ar = ph[u] - hdr->cab[rh] + (rv[u] - oh[u]);
-                    radr[la] = map_rank(cta_addr(res + ar), rh);
+                    const unsigned wd = pack_adr(rh, kh[u] - H()->klo[rh], ph[u] - H()->cab[rh] + (rv[u] - oh[u]));
+                    if (rh == rank) {
+                        adr[la] = wd;
+                    } else {
+                        const int sl = atomicAdd(&H()->nrem, 1);
+                        adr[la] = pack_adr((rank + 1) & (kClusterMax - 1), 0, 0) | (unsigned)sl;
+                        if (sl < nrcap) rw[sl] = wd;
+                    }
                     const int c0 = cj[u] + cr[u];   // res(a) + res(reverse of a), fixed
                     if (nar) {
                         res[la] = r0[u] | (c0 << 16);
@@ -436,17 +582,21 @@ struct ClusterFlow {
                 }
             }
         }
-        nremote = (int)__reduce_add_sync(FULL, (unsigned)nremote);
-        if ((threadIdx.x & 31) == 0 && nremote) atomicAddLL(&w.ctl->cl_remote, (long long)nremote);
         if (threadIdx.x == 0) {
-            hdr->nv = nv;
+            H()->nv = nv;
             const int a1 = khi < V ? __ldcg(&pacs[khi]) : A;
             cofs[nv] = a1 - abase;
-            hdr->na = a1 - abase;
-            if (rank == 0) { hdr->cnt[0] = hdr->cnt[1] = hdr->cnt[2] = 0; hdr->err = 0; }
+            H()->na = a1 - abase;
+            if (rank == 0) { H()->cnt[0] = H()->cnt[1] = H()->cnt[2] = 0; H()->err = 0; }
         }
-        rot = 0;
+        rot = arot = 0;
         sync();
+        const int nrem = H()->nrem;
+        if (cluster_any(nrem > nrcap)) return false;   // no room for the remote tables
+        if (threadIdx.x == 0 && nrem) atomicAddLL(&w.ctl->cl_remote, (long long)nrem);
+        for (int i = threadIdx.x; i < nrem; i += TPB)
+            rslot[i] = (unsigned short)adr_slot((unsigned)dsm_ld(map_rank(adr0 + 4 * adr_arc(rw[i]), adr_rank(rw[i]))));
+        sync();   // (no CTA sends into another's tables before it has read its slots)
         const int hmax = V + 2;
         mark(t1, T_CL_LOAD);
         // a maximum preflow is enough for the cut (see the grid-wide maxflow); the
@@ -466,7 +616,7 @@ struct ClusterFlow {
             mark(t1, T_CL_REACH);
             int open = 0;
             for (int lv = threadIdx.x; lv < nv; lv += TPB) open += rfl[lv] == 3;
-            if (cluster_sum(open) == 0) break;
+            if (!cluster_any(open)) break;
             if (attempt >= 16) {   // the same count in every CTA
                 if (rank == 0 && threadIdx.x == 0) fail(w.ctl, E_INTERNAL, 304);
                 break;
@@ -494,7 +644,7 @@ struct ClusterFlow {
         sync();
         // most balanced cut: SCCs of the residual graph on the vertices reached from
         // neither s nor t (lab, ex, fx are free now)
-        int *sc = fx;
+        const ShArr<int> sc = fx;
         if (w.pairs[p].mb) {
             scc_local(nv, V, sc);
         } else {
@@ -519,8 +669,8 @@ struct ClusterFlow {
     // successors).  sc: -2 outside X, else the root's union id.
     // V, the pair's vertex count, bounds the rounds: the same bound in every CTA, so
     // that every CTA leaves the loop after the same barrier.
-    __device__ void scc_local(int nv, int V, int *sc) {
-        int *col = lab, *done = ex;
+    __device__ void scc_local(int nv, int V, const ShArr<int> sc) {
+        const ShArr<int> col = lab, done = ex;
         for (int lv = threadIdx.x; lv < nv; lv += TPB) sc[lv] = rfl[lv] == 0 ? -1 : -2;
         sync();
         long long rounds = 0;
@@ -533,36 +683,34 @@ struct ClusterFlow {
                 cla[lv] = -1;
                 rem += un;
             }
-            if (cluster_sum(rem) == 0) break;
+            if (!cluster_any(rem)) break;
             if (++rounds > (long long)V + 1) {
                 if (rank == 0 && threadIdx.x == 0) fail(w.ctl, E_ITER, 303);
                 break;
             }
             // colours
-            const int lane = threadIdx.x & 31;
             for (;;) {
-                int nproc = 0;
+                bool any = false;
                 for (int k = 0; k < kScans; ++k) {
-                    for (int base = threadIdx.x - lane; base < nv; base += TPB) {
-                        const int lv = base + lane;
-                        int c = 0;
-                        bool fl = false;
-                        if (lv < nv && sc[lv] == -1) {
-                            c = *(volatile int *)&col[lv];
-                            fl = c < done[lv];
-                            if (fl) done[lv] = c;
-                        }
-                        nproc += fl;
-                        for_flagged(fl, [&](int src, int gl, int G) {
-                            const int cu = __shfl_sync(FULL, c, src < 0 ? 0 : src);
-                            if (src < 0) return;
-                            const int u = base + src, a1 = cofs[u + 1];
-                            for (int a = cofs[u] + gl; a < a1; a += G)
-                                if (rs(a) > 0) dsm_min(hadr[a], cu);   // col is lab
+                    const int n = collect(nv, [&](int lv) {
+                        return sc[lv] == -1 && *(volatile int *)&col[lv] < done[lv];
+                    });
+                    if (n == 0) break;
+                    any = true;
+                    each<4>(n, [&](int u, int gl) {
+                        // (one value for the vertex's lanes: it may drop meanwhile)
+                        const int cu = __shfl_sync(FULL, u >= 0 ? *(volatile int *)&col[u] : 0, 0, 4);
+                        if (u < 0) return;
+                        if (gl == 0) done[u] = cu;
+                        walk<4>(u, gl, [&](unsigned wd, int r, int) {
+                            if (r <= 0) return;
+                            if (local(wd)) atomicMin(&col[adr_vtx(wd)], cu);
+                            else enqueue(Q_MIN, adr_slot(wd), cu);   // (col is lab)
                         });
-                    }
+                    });
+                    flush();
                 }
-                if (cluster_sum(nproc) == 0) break;
+                if (!cluster_any(any)) break;
             }
             // roots, then members claim the vertices of their colour that reach them
             for (int lv = threadIdx.x; lv < nv; lv += TPB) {
@@ -571,38 +719,35 @@ struct ClusterFlow {
             }
             sync();
             for (;;) {
-                int nproc = 0;
+                bool any = false;
                 for (int k = 0; k < kScans; ++k) {
-                    for (int base = threadIdx.x - lane; base < nv; base += TPB) {
-                        const int lv = base + lane;
-                        int s = -1;
-                        bool fl = false;
-                        if (lv < nv && !done[lv]) {
-                            s = sc[lv];
-                            if (s == -1 && *(volatile int *)&cla[lv] == col[lv]) {
-                                s = col[lv];
-                                sc[lv] = s;
-                            }
-                            fl = s >= 0;
-                            if (fl) done[lv] = 1;
+                    const int n = collect(nv, [&](int lv) {
+                        return !done[lv] && (sc[lv] >= 0 || *(volatile int *)&cla[lv] == col[lv]);
+                    });
+                    if (n == 0) break;
+                    any = true;
+                    each<4>(n, [&](int u, int gl) {
+                        if (u < 0) return;
+                        const int su = sc[u] >= 0 ? sc[u] : col[u];   // (the same before and after the next line)
+                        if (gl == 0) {
+                            sc[u] = su;
+                            done[u] = 1;
                         }
-                        nproc += fl;
-                        for_flagged(fl, [&](int src, int gl, int G) {
-                            const int su = __shfl_sync(FULL, s, src < 0 ? 0 : src);
-                            if (src < 0) return;
-                            const int u = base + src, a1 = cofs[u + 1];
-                            for (int a = cofs[u] + gl; a < a1; a += G)
-                                if (cs(a) > rs(a)) dsm_max(hadr[a] + o_cla, su);
+                        walk<4>(u, gl, [&](unsigned wd, int r, int c) {
+                            if (c <= r) return;
+                            if (local(wd)) atomicMax(&cla[adr_vtx(wd)], su);
+                            else enqueue(Q_MAX, adr_slot(wd), su);
                         });
-                    }
+                    });
+                    flush();
                 }
-                if (cluster_sum(nproc) == 0) break;
+                if (!cluster_any(any)) break;
             }
         }
         if (rank == 0 && threadIdx.x == 0) atomicAdd(&w.ctl->scc_rounds, (int)rounds);
     }
 
-    static constexpr int kScans = 4;   // local scans between cluster barriers (relabel, reach)
+    static constexpr int kScans = 8;   // local scans between cluster barriers, at most (relabel, reach, SCCs)
     static constexpr int kMaxSweeps = 1024;   // sweeps of one wave (a bound; a wave ends when one moves nothing)
     static constexpr int kMaxLocalRounds = 4096;   // local rounds of one sweep (a bound)
 
@@ -610,7 +755,7 @@ struct ClusterFlow {
     // label correction pushed outward.  A vertex whose label dropped since it last
     // passed it on lowers the label of each v with a residual arc v -> u to its own
     // + 1 (an atomic min into v's CTA; the residual of v -> u is csum - res of
-    // u -> v) and publishes it to the arcs' copies.  Every CTA rescans its own
+    // u -> v).  Every CTA rescans its own
     // vertices kScans times between cluster barriers, without waiting for the
     // others; a barrier window in which no CTA had a vertex to pass on ends it
     // (every update sent before the window's barrier was seen in it), and the
@@ -624,42 +769,41 @@ struct ClusterFlow {
             lab[lv] = src ? 1 : hmax;
             rfl[lv] = hmax;
         }
-        const int na = hdr->na;
-        for (int a = threadIdx.x; a < na; a += TPB) hlab[a] = hmax;
         sync();
         long long arcs = 0;   // arcs this thread's vertices passed their labels along
         const int lane = threadIdx.x & 31;
         for (;;) {
-            int nproc = 0;
+            bool any = false;
             for (int k = 0; k < kScans; ++k) {
-                for (int base = threadIdx.x - lane; base < nv; base += TPB) {
-                    const int lv = base + lane;
-                    int L = 0;
-                    bool fr = false;
-                    if (lv < nv) {
-                        L = *(volatile int *)&lab[lv];
-                        fr = L < rfl[lv];
-                        if (fr) {
-                            rfl[lv] = L;
-                            arcs += cofs[lv + 1] - cofs[lv];
-                        }
+                const int n = collect(nv, [&](int lv) { return *(volatile int *)&lab[lv] < rfl[lv]; });
+                if (n == 0) break;
+                any = true;
+                auto pass_on = [&](auto G, int u, int gl) {
+                    // (one value for the vertex's lanes: it may drop meanwhile)
+                    const int Lu = __shfl_sync(FULL, u >= 0 ? *(volatile int *)&lab[u] : 0, 0, G());
+                    if (u < 0) return;
+                    if (gl == 0) {
+                        rfl[u] = Lu;
+                        arcs += cofs[u + 1] - cofs[u];
                     }
-                    nproc += fr;
-                    for_flagged(fr, [&](int src, int gl, int G) {
-                        const int Lu = __shfl_sync(FULL, L, src < 0 ? 0 : src);
-                        if (src < 0) return;
-                        const int u = base + src, a1 = cofs[u + 1];
-                        for (int a = cofs[u] + gl; a < a1; a += G) {
-                            dsm_st(radr[a] + o_hlab, Lu);
-                            if (cs(a) > rs(a)) dsm_min(hadr[a], Lu + 1);
-                        }
+                    walk<G()>(u, gl, [&](unsigned wd, int r, int c) {
+                        if (c <= r) return;
+                        if (local(wd)) atomicMin(&lab[adr_vtx(wd)], Lu + 1);
+                        else enqueue(Q_MIN, adr_slot(wd), Lu + 1);
                     });
-                }
+                };
+                if (n <= TPB / 8) each<8>(n, [&](int u, int gl) { pass_on(Int<8>(), u, gl); });
+                else each<4>(n, [&](int u, int gl) { pass_on(Int<4>(), u, gl); });
+                flush();
             }
-            if (cluster_sum(nproc) == 0) break;
+            if (!cluster_any(any)) break;
         }
         for (int o = 16; o > 0; o >>= 1) arcs += __shfl_xor_sync(FULL, arcs, o);
         if (lane == 0 && arcs) atomicAddLL(&w.ctl->gr_arcs, arcs);
+        // the copies of remote labels (the barrier: none is read after its owner lifts it)
+        const int nrem = H()->nrem;
+        for (int i = threadIdx.x; i < nrem; i += TPB) rg[i] = dsm_ld(head_at(rw[i]));
+        sync();
         int top = 0;
         if (want_top) {
             top = 1;
@@ -669,6 +813,16 @@ struct ClusterFlow {
         }
         if (rank == 0 && threadIdx.x == 0) atomicAddLL(&w.ctl->timers[T_CL_RELABEL], (long long)(globaltimer() - t_rel));
         return top;
+    }
+
+    // d along an arc in a wave: its reverse residual and its head's excess grow
+    __device__ __forceinline__ void give(unsigned wd, int d) {
+        if (local(wd)) {
+            atomicAdd(&res[adr_arc(wd)], d);
+            atomicAdd(&ex[adr_vtx(wd)], d);
+        } else {
+            send(Q_PUSH, adr_slot(wd), d);
+        }
     }
 
     // One level-synchronous wave (the waves before the pulses): the levels from the
@@ -688,22 +842,21 @@ struct ClusterFlow {
                 } else {
                     const int a1 = cofs[lv + 1];
                     for (int a = cofs[lv]; a < a1 && e > 0; a += U) {
-                        int r[U], hr[U], l[U];
+                        int r[U], l[U];
+                        unsigned hr[U];
 #pragma unroll
                         for (int u = 0; u < U; ++u) {
                             r[u] = a + u < a1 ? rs(a + u) : 0;
-                            hr[u] = a + u < a1 ? (int)hadr[a + u] : 0;
-                            l[u] = a + u < a1 ? hlab[a + u] : -1;
+                            hr[u] = a + u < a1 ? adr[a + u] : 0u;
                         }
 #pragma unroll
-                        for (int u = 0; u < U; ++u) l[u] = r[u] > 0 ? l[u] : -1;
+                        for (int u = 0; u < U; ++u) l[u] = r[u] > 0 ? head_label(hr[u]) : -1;
 #pragma unroll
                         for (int u = 0; u < U; ++u) {
                             if (e > 0 && l[u] == L - 1) {
                                 const int d = e < r[u] ? e : r[u];
                                 set_rs(a + u, r[u] - d);
-                                dsm_add(radr[a + u], d);
-                                dsm_add((unsigned)hr[u] + o_ex, d);
+                                give(hr[u], d);
                                 e -= d;
                             }
                         }
@@ -729,11 +882,10 @@ struct ClusterFlow {
     // pushes at most what it read; others only add).  Every push lowers the sum of
     // excess times label, so the rounds and the sweeps end.
     __device__ void wave_levels(int ph, int nv, int top) {
-        const unsigned own_lo = map_rank(cta_addr(lab), rank), own_hi = own_lo + 4u * (unsigned)nv;
         for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
             int moved = 0;
             for (int round = 0; round < kMaxLocalRounds; ++round) {
-                int local = 0;
+                int landed = 0;
                 for (int lv = threadIdx.x; lv < nv; lv += TPB) {
                     const int L = lab[lv];
                     if (L < 1 || L > top) continue;
@@ -751,21 +903,19 @@ struct ClusterFlow {
 #pragma unroll
                             for (int u = 0; u < U; ++u) {
                                 r[u] = a + u < a1 ? rs(a + u) : 0;
-                                hr[u] = a + u < a1 ? hadr[a + u] : 0u;
-                                l[u] = a + u < a1 ? hlab[a + u] : -1;
+                                hr[u] = a + u < a1 ? adr[a + u] : 0u;
                             }
 #pragma unroll
-                            for (int u = 0; u < U; ++u) l[u] = r[u] > 0 ? l[u] : -1;
+                            for (int u = 0; u < U; ++u) l[u] = r[u] > 0 ? head_label(hr[u]) : -1;
 #pragma unroll
                             for (int u = 0; u < U; ++u) {
                                 if (e > 0 && l[u] == L - 1) {
                                     const int d = e < r[u] ? e : r[u];
                                     set_rs(a + u, r[u] - d);
-                                    dsm_add(radr[a + u], d);
-                                    dsm_add(hr[u] + o_ex, d);
+                                    give(hr[u], d);
                                     e -= d;
                                     sent += d;
-                                    local |= hr[u] >= own_lo && hr[u] < own_hi;
+                                    landed |= local(hr[u]);
                                 }
                             }
                         }
@@ -775,9 +925,9 @@ struct ClusterFlow {
                         ++moved;
                     }
                 }
-                if (!__syncthreads_or(local)) break;
+                if (!__syncthreads_or(landed)) break;
             }
-            if (cluster_sum(moved) == 0) break;
+            if (!cluster_any(moved)) break;
         }
     }
 
@@ -790,7 +940,7 @@ struct ClusterFlow {
             const int top = relabel(ph, nv, hmax, true);
             int act = 0;
             for (int lv = threadIdx.x; lv < nv; lv += TPB) act += ex[lv] > 0 && lab[lv] < hmax;
-            if (cluster_sum(act) == 0) break;
+            if (!cluster_any(act)) break;
             if (++waves > w.pulse_cap) return false;
             wave_levels(ph, nv, top);
         }
@@ -801,7 +951,154 @@ struct ClusterFlow {
         return true;
     }
 
-    // Lock-free pulses (push to the lowest residual neighbour or relabel) until no
+    // One vertex holding excess, G lanes: lift it just above its lowest residual neighbour if
+    // it is not, push along the arc to that neighbour, up to `iters` times or until the excess
+    // is gone.  Copies of remote labels may lag; they never run ahead of the label, and
+    // labels only rise between exact relabels, so a lagging copy only makes a push look
+    // admissible that is not -- capacities and excesses stay exact, and a phase ends only once
+    // exact labels (phase 1) or the residual sets (phase 0) show that no excess can still
+    // reach its target.  Returns (on the vertices' first lanes) whether the vertex pushed along
+    // an arc or still holds excess that may move.  All lanes of a warp call it (u < 0: none).
+    // The passes are bound by the instructions of a visit (four warps a scheduler, each some
+    // hundreds): pushing along all arcs to the lowest label at once, their shares by a prefix
+    // sum, took three times as many an iteration.
+    template <int G>
+    __device__ __forceinline__ bool discharge(int ph, int u, int gl, int hmax, int iters) {
+        int e = 0, f = 0, h = hmax, sent = 0, a0 = 0, deg = 0;
+        bool border = false, pushed = false;
+        if (u >= 0) {
+            e = *(volatile int *)&ex[u];
+            f = fx[u];
+            h = lab[u];
+            a0 = cofs[u];
+            deg = cofs[u + 1] - a0;
+            border = bord[u] == (ph ? 1 : 2);
+        }
+        e = __shfl_sync(FULL, e, 0, G);   // (it may grow meanwhile)
+        __syncwarp();
+        if (border) {   // the arc to the target
+            sent = ph ? min(e, f) : e;
+            if (gl == 0) fx[u] = ph ? f - sent : f + sent;
+            e -= sent;
+        }
+        const int longest = (int)__reduce_max_sync(FULL, (unsigned)(e > 0 ? deg : 0));
+        if (longest <= 16) discharge_row<G, 16 / G>(a0, deg, u, gl, hmax, iters, h, e, sent, pushed);
+        else if (longest <= 32) discharge_row<G, 32 / G>(a0, deg, u, gl, hmax, iters, h, e, sent, pushed);
+        else discharge_long<G>(a0, deg, u, gl, hmax, iters, h, e, sent, pushed);
+        if (gl != 0 || u < 0) return false;
+        if (sent) atomicSub(&ex[u], sent);
+        return pushed || (e > 0 && h < hmax);
+    }
+
+    // the lowest of a vertex's G lanes
+    template <int G>
+    __device__ __forceinline__ int lowest(int x) const {
+#pragma unroll
+        for (int d = G / 2; d > 0; d >>= 1) x = min(x, __shfl_xor_sync(FULL, x, d));
+        return x;
+    }
+    __device__ __forceinline__ void push_arc(int a, unsigned wd, int d) {
+        atomicSub(&res[a], d);
+        if (local(wd)) {
+            atomicAdd(&res[adr_arc(wd)], d);
+            atomicAdd(&ex[adr_vtx(wd)], d);
+        } else {
+            enqueue(Q_PUSH, adr_slot(wd), d);
+        }
+    }
+    __device__ __forceinline__ void publish(int a0, int na, int gl, int G, int h) {
+#pragma unroll 1
+        for (int a = gl; a < na; a += G) {
+            const unsigned wd = adr[a0 + a];
+            if (!local(wd)) enqueue(Q_LABEL, adr_slot(wd), h);
+        }
+    }
+
+    // rows of up to G R <= 32 arcs: the lanes keep label << 5 | place for their residual arcs
+    template <int G, int R>
+    __device__ __forceinline__ void discharge_row(int a0, int deg, int u, int gl, int hmax, int iters, int &h, int &e,
+                                                  int &sent, bool &pushed) {
+        int key[R];
+        unsigned wd[R];
+        const int h0 = h, na = e > 0 ? deg : 0;
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            const bool v = gl + G * i < na;
+            wd[i] = v ? adr[a0 + gl + G * i] : 0u;
+            key[i] = v ? rs(a0 + gl + G * i) : 0;
+        }
+#pragma unroll
+        for (int i = 0; i < R; ++i) key[i] = key[i] > 0 ? head_label(wd[i]) << 5 | (gl + G * i) : INT_MAX;
+        for (int it = 0; it < iters; ++it) {
+            const bool go = e > 0 && h < hmax;
+            if (!__any_sync(FULL, go)) break;
+            int k = INT_MAX;
+#pragma unroll
+            for (int i = 0; i < R; ++i) k = min(k, key[i]);
+            k = lowest<G>(k);
+            const int hm = k >> 5, at = k & 31;
+            if (go && h <= hm) h = hm >= hmax - 1 ? hmax : hm + 1;
+            const bool push = go && h < hmax;
+            int d = 0, r = 0;
+            if (push) {
+                r = rs(a0 + at);
+                d = min(e, r);
+            }
+            d = __shfl_sync(FULL, d, 0, G);   // (a residual may grow meanwhile)
+            if (push) {
+                if (gl == 0) push_arc(a0 + at, adr[a0 + at], d);
+#pragma unroll
+                for (int i = 0; i < R; ++i) key[i] = key[i] == k && d < e ? INT_MAX : key[i];   // saturated
+                pushed = true;
+                sent += d;
+                e -= d;
+            }
+        }
+        if (h != h0) {
+            if (gl == 0) lab[u] = h;
+            publish(a0, na, gl, G, h);
+        }
+    }
+
+    // longer rows: the same, an iteration reading its arcs again
+    template <int G>
+    __device__ __forceinline__ void discharge_long(int a0, int deg, int u, int gl, int hmax, int iters, int &h, int &e,
+                                                   int &sent, bool &pushed) {
+        const int h0 = h, na = e > 0 ? deg : 0;
+        for (int it = 0; it < iters; ++it) {
+            const bool go = e > 0 && h < hmax;
+            if (!__any_sync(FULL, go)) break;
+            int hm = INT_MAX, at = INT_MAX;
+            if (go)
+                for (int a = gl; a < deg; a += G) {
+                    const int l = rs(a0 + a) > 0 ? head_label(adr[a0 + a]) : INT_MAX;
+                    if (l < hm) {
+                        hm = l;
+                        at = a;
+                    }
+                }
+            const int mine = hm;
+            hm = lowest<G>(hm);
+            at = lowest<G>(mine == hm ? at : INT_MAX);
+            if (go && h <= hm) h = hm >= hmax - 1 ? hmax : hm + 1;
+            const bool push = go && h < hmax;
+            int d = 0;
+            if (push) d = min(e, rs(a0 + at));
+            d = __shfl_sync(FULL, d, 0, G);
+            if (push) {
+                if (gl == 0) push_arc(a0 + at, adr[a0 + at], d);
+                pushed = true;
+                sent += d;
+                e -= d;
+            }
+        }
+        if (h != h0) {
+            if (gl == 0) lab[u] = h;
+            publish(a0, na, gl, G, h);
+        }
+    }
+
+    // Lock-free pulses (every vertex holding excess is discharged) until no
     // vertex with excess has a label below hmax; phase 1 returns excess to s.
     // certify: end only after an exact relabel confirms that no excess can move
     // (phase 1; phase 0 is checked by the residual sets instead).
@@ -821,55 +1118,25 @@ struct ClusterFlow {
             int act = 0;
             for (int pass = 0; pass < w.passes; ++pass) {
                 const bool last = pass + 1 == w.passes;
-                for (int lv = threadIdx.x; lv < nv; lv += TPB) {
-                    int e = *(volatile int *)&ex[lv];
-                    if (e <= 0) continue;
-                    int h = lab[lv];
-                    if (h >= hmax) continue;
-                    const int a0 = cofs[lv], a1 = cofs[lv + 1];
-                    const unsigned char bd = bord[lv];
-                    for (int it = 0; it < w.inner; ++it) {
-                        int hmin, best;
-                        lowest(a0, a1, hmin, best);
-                        if (ph ? (bd == 1 && fx[lv] > 0) : (bd == 2)) { hmin = 0; best = -2; }
-                        if (best == -1) { h = hmax; set_label(lv, h); break; }
-                        if (h > hmin) {
-                            int d;
-                            if (best == -2) {
-                                if (!ph) { d = e; fx[lv] += d; }
-                                else { d = e < fx[lv] ? e : fx[lv]; fx[lv] -= d; }
-                            } else {
-                                const int r = rs(best);
-                                d = e < r ? e : r;
-                                const unsigned hh = hadr[best], rv = radr[best];
-                                atomicSub(&res[best], d);
-                                dsm_add(rv, d);
-                                dsm_add(hh + o_ex, d);
-                                if (last) ++act;
-                            }
-                            atomicSub(&ex[lv], d);
-                            e -= d;
-                            if (e == 0) break;
-                        } else {
-                            h = hmin + 1;
-                            if (h >= hmax) h = hmax;
-                            set_label(lv, h);
-                            if (h >= hmax) break;
-                        }
-                    }
-                    if (last && e > 0 && h < hmax) ++act;
-                }
+                const int n = collect(nv, [&](int lv) { return lab[lv] < hmax && *(volatile int *)&ex[lv] > 0; });
+                auto visit = [&](auto G, int u, int gl) {
+                    const bool on = discharge<G()>(ph, u, gl, hmax, w.inner);
+                    if (last) act += on;
+                };
+                if (n <= TPB / 8) each<8>(n, [&](int u, int gl) { visit(Int<8>(), u, gl); });
+                else each<4>(n, [&](int u, int gl) { visit(Int<4>(), u, gl); });
+                flush();
             }
             ++pulses;
             ++since;
-            const int a = cluster_sum(act);
+            const bool a = cluster_any(act);
             if (pulses > w.pulse_cap) return false;
-            if (a == 0) {
+            if (!a) {
                 // pushes of earlier passes may land after their target was scanned
                 int left = 0;
                 for (int lv = threadIdx.x; lv < nv; lv += TPB)
                     left += ex[lv] > 0 && lab[lv] < hmax;
-                if (cluster_sum(left) == 0) {
+                if (!cluster_any(left)) {
                     if (!certify) break;
                     // Nothing can move by the current labels.  Exact labels decide:
                     // the phase ends only if no vertex with excess can reach its
@@ -881,7 +1148,7 @@ struct ClusterFlow {
                     left = 0;
                     for (int lv = threadIdx.x; lv < nv; lv += TPB)
                         left += ex[lv] > 0 && lab[lv] < hmax;
-                    if (cluster_sum(left) == 0) break;
+                    if (!cluster_any(left)) break;
                     continue;
                 }
             }
@@ -909,12 +1176,12 @@ struct ClusterFlow {
     // Returns the vertices lifted (cluster-wide).
     __device__ int gap(int nv, int hmax) {
         const int nwords = (hmax + 31) >> 5;
-        if (nwords > hdr->nvcap) return 0;   // (tiny ranges: the bitmap does not fit; the same in every CTA)
-        unsigned *bm = reinterpret_cast<unsigned *>(cla);
+        if (nwords > H()->nvcap) return 0;   // (tiny ranges: the bitmap does not fit; the same in every CTA)
+        const ShArr<unsigned> bm{cla.o};
         if (rank == 0)
             for (int i = threadIdx.x; i < nwords; i += TPB) bm[i] = 0u;
         sync();
-        const unsigned bm0 = map_rank(cta_addr(bm), 0);
+        const unsigned bm0 = map_rank(cta_addr(bm.ptr()), 0);
         int top = 0;
         for (int lv = threadIdx.x; lv < nv; lv += TPB) {
             const int h = lab[lv];
@@ -941,10 +1208,14 @@ struct ClusterFlow {
         for (int lv = threadIdx.x; lv < nv; lv += TPB) {
             const int h = lab[lv];
             if (h > h0 && h < hmax) {
-                set_label(lv, hmax);
+                lab[lv] = hmax;
+                const int a1 = cofs[lv + 1];
+                for (int a = cofs[lv]; a < a1; ++a)
+                    if (!local(adr[a])) enqueue(Q_LABEL, adr_slot(adr[a]), hmax);
                 ++lifted;
             }
         }
+        flush();
         lifted = cluster_sum(lifted);
         if (rank == 0 && threadIdx.x == 0) {
             atomicAddLL(&w.ctl->gaps, 1);
@@ -966,32 +1237,33 @@ struct ClusterFlow {
             lab[lv] = 0;
         }
         sync();
-        const int lane = threadIdx.x & 31;
         for (;;) {
-            int nproc = 0;
+            bool any = false;
             for (int k = 0; k < kScans; ++k) {
-                for (int base = threadIdx.x - lane; base < nv; base += TPB) {
-                    const int lv = base + lane;
-                    int nw = 0;
-                    if (lv < nv) {
-                        const int f = *(volatile int *)&rfl[lv], dn = lab[lv];
-                        nw = f & ~dn;
-                        if (nw) lab[lv] = dn | nw;
+                const int n = collect(nv, [&](int lv) { return (*(volatile int *)&rfl[lv] & ~lab[lv]) != 0; });
+                if (n == 0) break;
+                any = true;
+                each<4>(n, [&](int u, int gl) {
+                    int nw = 0, f = 0;
+                    if (u >= 0) {
+                        f = *(volatile int *)&rfl[u];
+                        nw = f & ~lab[u];
                     }
-                    nproc += nw != 0;
-                    for_flagged(nw != 0, [&](int src, int gl, int G) {
-                        const int nwu = __shfl_sync(FULL, nw, src < 0 ? 0 : src);
-                        if (src < 0) return;
-                        const int u = base + src, a1 = cofs[u + 1];
-                        for (int a = cofs[u] + gl; a < a1; a += G) {
-                            const int r = rs(a);
-                            const int bits = ((nwu & 1) && r > 0 ? 1 : 0) | ((nwu & 2) && cs(a) > r ? 2 : 0);
-                            if (bits) dsm_or(hadr[a] + o_rfl, bits);
-                        }
+                    // (the vertex's lanes may have read different bits: all pass on all of them)
+                    nw |= __shfl_xor_sync(FULL, nw, 1);
+                    nw |= __shfl_xor_sync(FULL, nw, 2);
+                    if (u < 0) return;
+                    if (gl == 0) lab[u] |= nw;
+                    walk<4>(u, gl, [&](unsigned wd, int r, int c) {
+                        const int bits = ((nw & 1) && r > 0 ? 1 : 0) | ((nw & 2) && c > r ? 2 : 0);
+                        if (!bits) return;
+                        if (local(wd)) atomicOr(&rfl[adr_vtx(wd)], bits);
+                        else enqueue(Q_OR, adr_slot(wd), bits);
                     });
-                }
+                });
+                flush();
             }
-            if (cluster_sum(nproc) == 0) break;
+            if (!cluster_any(any)) break;
         }
     }
 };
