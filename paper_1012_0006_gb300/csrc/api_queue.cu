@@ -112,7 +112,7 @@ fr_status ensure_queue(fr_ctx *ctx, int ctas, int clusters, int n, int nnz, int 
     ctx->q_np = pp;
     ctx->q_nu = c.nu; ctx->q_mu = c.mu; ctx->q_vq = c.vq;
     char *p = reinterpret_cast<char *>(ctx->q_mem);
-    ctx->q_ticket = take<int>(p, 1);
+    ctx->q_ticket = take<int>(p, 2);
     ctx->q_gabort = take<int>(p, 1);
     ctx->q_prev = take<int>(p, 2LL * pp);
     ctx->q_crank = take<int>(p, mm);
@@ -273,6 +273,7 @@ fr_status run_queue_sweep(fr_ctx *ctx, const fr_graph *g, int32_t *part, const B
     q.slots = ctx->q_slots;
     q.np = pl.np;
     q.ticket = ctx->q_ticket;
+    q.votes = q.wt.flow_sched == 0 ? ctx->q_ticket + 1 : nullptr;
     q.prev = ctx->q_prev;
     q.gabort = ctx->q_gabort;
     q.wait_ns = kWaitNs;
@@ -281,7 +282,7 @@ fr_status run_queue_sweep(fr_ctx *ctx, const fr_graph *g, int32_t *part, const B
         CK(launch_fill_pairs(ctx->pairs, ctx->pair_a, ctx->pair_b, pl.np, 0, opt->mb ? 1 : 0, pl.Ubase, ctx->stream));
         CK(cudaMemsetAsync(ctx->sides, 0, sizeof(SideDev) * 2 * (size_t)pl.np, ctx->stream));
         CK(cudaMemsetAsync(ctx->pacc, 0, sizeof(PairAcc) * (size_t)pl.np, ctx->stream));
-        CK(cudaMemsetAsync(ctx->q_ticket, 0, sizeof(int), ctx->stream));
+        CK(cudaMemsetAsync(ctx->q_ticket, 0, 2 * sizeof(int), ctx->stream));   // (and the votes)
         CK(cudaMemsetAsync(ctx->q_gabort, 0, sizeof(int), ctx->stream));
         CK(cudaMemsetAsync(ctx->q_ctls, 0, sizeof(fr_ctx::QCtl) * (size_t)clusters, ctx->stream));
         CK(cudaMemsetAsync(ctx->q_stats, 0, 4 * sizeof(long long) * (size_t)clusters, ctx->stream));

@@ -187,6 +187,7 @@ struct Work {
     int narrow;                  // 1: every arc capacity < 2^15 (cluster kernel packs residual and capacity sum)
     int pre_waves;               // cluster pulses: waves by levels before the first pulse
     int gap_interval;            // pulses between gap checks of push-relabel (0: none)
+    int *wave_votes;             // queue sweep: this pair starts with a wave, and tells whether it paid (NULL: not)
     unsigned long long seed;
     long long pulse_cap;
     int *crank;                  // per graph arc: rank among its row's corridor arcs (NULL: outs holds it)

@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(TPB, 1) queue_kernel(QueueArgs q, size_t smem_
     extern __shared__ __align__(16) char csmem[];
     __shared__ Work s_w;
     __shared__ __align__(16) int s_side[32];   // the step phases' per-side state (two sides)
-    __shared__ int s_grab[2];
+    __shared__ int s_grab[2], s_try[2];
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank(), C = (int)cl.num_blocks();
     const QSlot &S = q.slots[blockIdx.x / C];
@@ -91,9 +91,12 @@ __global__ void __launch_bounds__(TPB, 1) queue_kernel(QueueArgs q, size_t smem_
                 }
             }
             s_grab[it & 1] = j;
+            // every eighth pair tries the wave, and any while it has paid more often than not
+            s_try[it & 1] = q.votes && ((j & 7) == 0 || *(volatile int *)q.votes > 0);
         }
         cl.sync();
         const int j = *(volatile int *)cl.map_shared_rank(&s_grab[it & 1], 0);
+        const bool try_wave = *(volatile int *)cl.map_shared_rank(&s_try[it & 1], 0) != 0;
         if (j >= q.np) break;
         const PairDev P = q.wt.pairs[j];
         if (threadIdx.x == 0) {
@@ -118,6 +121,7 @@ __global__ void __launch_bounds__(TPB, 1) queue_kernel(QueueArgs q, size_t smem_
             w.cl_tier = 0;
             w.list_ids = 1;
             w.gabort = q.gabort;
+            w.wave_votes = try_wave ? q.votes : nullptr;
             s_w = w;
             g_nsync = 0;
         }

@@ -39,6 +39,8 @@ struct QueueArgs {
     const QSlot *slots;   // [clusters]
     int np;               // pairs of the sweep, in round order
     int *ticket;          // next pair to take (zero before the launch)
+    int *votes;           // pairs whose flow started with a wave that paid, less those it did not pay
+                          // (zero before the launch; NULL: no pair does)
     const int *prev;      // [2 np]: the last earlier pair that shares block a (b), or -1
     int *gabort;          // 0, E_MISFIT (run the sweep round by round instead), or an error code
     unsigned long long wait_ns;   // bound of one wait for a dependency (then E_ABORT)
