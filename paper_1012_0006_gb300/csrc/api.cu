@@ -736,41 +736,68 @@ static fr_status run_pair_iteration(fr_ctx *ctx, const fr_graph *g, int32_t *par
                                     long long Ubase, long long Lmax, long long W, const fr_options *opt,
                                     IterOut *o) {
     const int mb = opt && opt->mb ? 1 : 0;
+    // corridor estimate: two sides of about (Ubase - W/k) weight each
+    const double avgc = std::max(1.0, (double)W / g->n);
+    const long long est = std::max<long long>(1, (long long)(2.0 * std::max(0LL, Ubase - W / k) / avgc));
+    char *h = ctx->h_stage + 2048;
+    auto out = [&](const Ctl &ctl) {
+        const PairAcc &A = *reinterpret_cast<PairAcc *>(h);
+        const SideDev *S = reinterpret_cast<SideDev *>(h + 512);
+        o->ctl = ctl;
+        o->flow = A.flow;
+        o->oldcut = A.oldcut;
+        o->newcut = A.oldcut + A.dcut;
+        o->cA = S[0].cw;
+        o->cB = S[1].cw;
+        o->nA = S[0].cw + A.dwA;
+        o->nB = S[1].cw - A.dwA;
+        o->nc = A.nc;
+        o->m = A.m;
+        o->accept = A.accept;
+        o->feasible = A.feasible;
+    };
+    // one launch of one cluster where the corridor fits
+    const int tq = queue_round_size(ctx, 1, est, (double)g->nnz / g->n, opt);
+    if (tq >= 0) {
+        PairDev *hp = reinterpret_cast<PairDev *>(ctx->h_stage + 1024);
+        hp->g = 0; hp->a = a; hp->b = b; hp->mb = mb; hp->Ubase = Ubase;
+        CK(cudaMemcpyAsync(ctx->pairs, hp, sizeof(PairDev), cudaMemcpyHostToDevice, ctx->stream));
+        CK(cudaMemsetAsync(ctx->sides, 0, 2 * sizeof(SideDev), ctx->stream));
+        CK(cudaMemsetAsync(ctx->pacc, 0, sizeof(PairAcc), ctx->stream));
+        RoundQueue rq;
+        fr_status sq = enqueue_round_queue(ctx, g, part, k, 1, Lmax, opt, tq, &rq);
+        if (sq != FR_OK) return sq;
+        if (rq.queued) {
+            CK(cudaMemcpyAsync(h, ctx->pacc, sizeof(PairAcc), cudaMemcpyDeviceToHost, ctx->stream));
+            CK(cudaMemcpyAsync(h + 512, ctx->sides, 2 * sizeof(SideDev), cudaMemcpyDeviceToHost, ctx->stream));
+            CK(cudaStreamSynchronize(ctx->stream));
+            sq = finish_round_queue(ctx, g, part, k, "fr_refine_pair", &rq);
+            if (sq != FR_OK) { o->ctl = rq.ctl; return sq; }
+            if (rq.queued) {
+                out(rq.ctl);
+                return FR_OK;
+            }
+        }
+    }
     fr_status st = setup_single(ctx, g, part, k, a, b, Ubase, Lmax, mb);
     if (st != FR_OK) return st;
     Work w = make_work(ctx, 0, 0, 1, g->n, opt);
     const int tpb = choose_tpb(ctx, opt);
-    // corridor estimate: two sides of about (Ubase - W/k) weight each
-    const double avgc = std::max(1.0, (double)W / g->n);
-    const long long est = std::max<long long>(1, (long long)(2.0 * std::max(0LL, Ubase - W / k) / avgc));
     const int grid = choose_grid(ctx, opt, tpb, 2, est);
     CK(launch_scan_list(w, 0, ctx->stream));
     CK(launch_round(ctx, w, grid, tpb, ctx->stream, nullptr, est, (double)g->nnz / g->n,
                     opt && opt->cluster_ctas ? opt->cluster_ctas : ctx->tune_ctas));
-    char *h = ctx->h_stage + 2048;
     CK(cudaMemcpyAsync(h, ctx->pacc, sizeof(PairAcc), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaMemcpyAsync(h + 512, ctx->sides, 2 * sizeof(SideDev), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaMemcpyAsync(h + 1024, ctx->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    const PairAcc &A = *reinterpret_cast<PairAcc *>(h);
-    const SideDev *S = reinterpret_cast<SideDev *>(h + 512);
     o->ctl = *reinterpret_cast<Ctl *>(h + 1024);
     st = status_from_ctl(ctx, o->ctl, "fr_refine_pair");
     if (st != FR_OK) {
         reset_idle(ctx);
         return st;
     }
-    o->flow = A.flow;
-    o->oldcut = A.oldcut;
-    o->newcut = A.oldcut + A.dcut;
-    o->cA = S[0].cw;
-    o->cB = S[1].cw;
-    o->nA = S[0].cw + A.dwA;
-    o->nB = S[1].cw - A.dwA;
-    o->nc = A.nc;
-    o->m = A.m;
-    o->accept = A.accept;
-    o->feasible = A.feasible;
+    out(o->ctl);
     return FR_OK;
 }
 

@@ -81,7 +81,6 @@ fr_status run_pairs_step(fr_ctx *ctx, const fr_graph *g, int32_t *part, int32_t 
     CK(cudaMemsetAsync(ctx->ctl, 0, sizeof(Ctl), ctx->stream));
     CK(cudaMemsetAsync(ctx->sides, 0, sizeof(SideDev) * 2 * P, ctx->stream));
     CK(cudaMemsetAsync(ctx->pacc, 0, sizeof(PairAcc) * P, ctx->stream));
-    CK(cudaMemsetAsync(ctx->hist, 0, sizeof(long long) * 3 * 2 * (size_t)P * kHistBins, ctx->stream));
     Work w = make_work(ctx, 0, 0, P, g->n, opt);
     const int tpb = choose_tpb(ctx, opt);
     const double avgc = std::max(1.0, (double)W / g->n);
@@ -96,9 +95,18 @@ fr_status run_pairs_step(fr_ctx *ctx, const fr_graph *g, int32_t *part, int32_t 
         int nf = 0;
         CK(launch_fm(w, fm_view(ctx, 0, opt), k, ctx->sms, ctx->stream, &nf));
     }
-    CK(launch_scan_list(w, 0, ctx->stream));
-    CK(launch_round(ctx, w, grid, tpb, ctx->stream, nullptr, emax, (double)g->nnz / g->n,
-                    opt->cluster_ctas ? opt->cluster_ctas : ctx->tune_ctas));
+    // one launch of clusters where the corridors fit, else the round's own sequence
+    RoundQueue rq;
+    const int tq = queue_round_size(ctx, P, emax, (double)g->nnz / g->n, opt);
+    if (tq >= 0 && (st = enqueue_round_queue(ctx, g, part, k, P, Lmax, opt, tq, &rq)) != FR_OK) return st;
+    auto own_launches = [&]() -> fr_status {
+        CK(cudaMemsetAsync(ctx->hist, 0, sizeof(long long) * 3 * 2 * (size_t)P * kHistBins, ctx->stream));
+        CK(launch_scan_list(w, 0, ctx->stream));
+        CK(launch_round(ctx, w, grid, tpb, ctx->stream, nullptr, emax, (double)g->nnz / g->n,
+                        opt->cluster_ctas ? opt->cluster_ctas : ctx->tune_ctas));
+        return FR_OK;
+    };
+    if (!rq.queued && (st = own_launches()) != FR_OK) return st;
     PairAcc *ha = reinterpret_cast<PairAcc *>(ctx->h_stage + (kHostStage / 2));
     SideDev *hsd = reinterpret_cast<SideDev *>(ha + P);
     Ctl *hc = reinterpret_cast<Ctl *>(hsd + 2 * P);
@@ -108,15 +116,32 @@ fr_status run_pairs_step(fr_ctx *ctx, const fr_graph *g, int32_t *part, int32_t 
         return FR_ERR_TOO_LARGE;
     }
     if (fm_first) CK(cudaMemcpyAsync(hf, ctx->fm.res, sizeof(FmRes) * P, cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaMemcpyAsync(ha, ctx->pacc, sizeof(PairAcc) * P, cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaMemcpyAsync(hsd, ctx->sides, sizeof(SideDev) * 2 * P, cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaMemcpyAsync(hc, ctx->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
+    auto read_back = [&]() -> fr_status {
+        CK(cudaMemcpyAsync(ha, ctx->pacc, sizeof(PairAcc) * P, cudaMemcpyDeviceToHost, ctx->stream));
+        CK(cudaMemcpyAsync(hsd, ctx->sides, sizeof(SideDev) * 2 * P, cudaMemcpyDeviceToHost, ctx->stream));
+        CK(cudaMemcpyAsync(hc, ctx->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, ctx->stream));
+        CK(cudaStreamSynchronize(ctx->stream));
+        return FR_OK;
+    };
+    if ((st = read_back()) != FR_OK) return st;
+    bool queued = rq.queued;
+    fr_status qst = FR_OK;
+    if (queued) {   // (ctx->ctl holds the FM step's errors, the clusters report their own)
+        qst = finish_round_queue(ctx, g, part, k, "fr_refine_active", &rq);
+        if (qst == FR_OK && !rq.queued && hc->error == 0) {   // a pair outgrew its cluster
+            queued = false;
+            CK(cudaMemsetAsync(ctx->sides, 0, sizeof(SideDev) * 2 * P, ctx->stream));
+            CK(cudaMemsetAsync(ctx->pacc, 0, sizeof(PairAcc) * P, ctx->stream));
+            if ((st = own_launches()) != FR_OK || (st = read_back()) != FR_OK) return st;
+        }
+    }
     st = status_from_ctl(ctx, *hc, "fr_refine_active");
+    if (st == FR_OK) st = qst;
     if (st != FR_OK) {
         reset_idle(ctx);
         return st;
     }
+    const Ctl &ran = queued ? rq.ctl : *hc;
     out.resize(P);
     for (int i = 0; i < P; ++i) {
         StepOut &o = out[i];
@@ -131,8 +156,8 @@ fr_status run_pairs_step(fr_ctx *ctx, const fr_graph *g, int32_t *part, int32_t 
         o.m = ha[i].m;
         o.accept = ha[i].accept;
         o.feasible = ha[i].feasible;
-        o.pulses = hc->pulses;
-        o.relabels = hc->relabels;
+        o.pulses = ran.pulses;
+        o.relabels = ran.relabels;
         if (fm_first) o.fm = hf[i];
         else memset(&o.fm, 0, sizeof(o.fm));
     }

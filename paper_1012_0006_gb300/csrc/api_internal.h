@@ -215,4 +215,20 @@ int queue_size_for(fr_ctx *ctx, const BatchPlan &pl, const fr_options *opt);
 // device errors restore part and return the error.
 fr_status run_queue_sweep(fr_ctx *ctx, const fr_graph *g, int32_t *part, const BatchPlan &pl, const fr_options *opt,
                           int t, float *ms, bool *ran, std::vector<fr::Ctl> *ctls);
+// One round of block-disjoint pairs as one launch of the queue kernel, each pair in a
+// cluster (ctx->pairs uploaded, ctx->sides and ctx->pacc cleared by the caller).
+// queue_round_size: index into kClusterSizes for P pairs whose largest corridor is estimated
+// at est vertices, or -1 where it does not apply.  enqueue: rq->queued = false if the arena
+// bound leaves no room.  After the caller synchronised the stream, finish reads what the
+// clusters reported: if a pair outgrew its cluster, part, the block weights and the idle
+// state are restored and rq->queued is false again (the caller runs the round's own launches).
+struct RoundQueue {
+    bool queued = false;
+    int clusters = 0;
+    fr::Ctl ctl = {};   // pulses, relabels, levels and SCC rounds over the clusters; the first error
+};
+int queue_round_size(fr_ctx *ctx, int P, long long est, double avg_degree, const fr_options *opt);
+fr_status enqueue_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int k, int P, long long Lmax,
+                              const fr_options *opt, int t, RoundQueue *rq);
+fr_status finish_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int k, const char *where, RoundQueue *rq);
 void destroy_graph_cache(fr_ctx *ctx);

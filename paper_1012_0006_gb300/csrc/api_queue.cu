@@ -25,6 +25,9 @@ constexpr double kRelTime[fr_ctx::kNumClusterSizes] = {1.25, 1.05, 1.0, 0.85, 0.
 // host staging offsets (the first megabytes of h_stage belong to the other paths)
 constexpr size_t kStageGraphs = 4u << 20;
 constexpr size_t kStagePrev = (4u << 20) + (64u << 10);
+// a round on the queue kernel (run_round_queue): descriptors, block weights, read-back
+constexpr size_t kStageRound = 6u << 20, kStageRoundW = (6u << 20) + (256u << 10),
+                 kStageRoundCtl = (6u << 20) + (512u << 10);
 constexpr unsigned long long kWaitNs = 10ull * 1000 * 1000 * 1000;   // one dependency wait, at most 10 s
 
 size_t al256(size_t b) { return (b + 255) / 256 * 256; }
@@ -100,14 +103,19 @@ fr_status ensure_queue(fr_ctx *ctx, int ctas, int clusters, int n, int nnz, int 
         ctx_error(ctx, "queue sweep workspace exceeds the arena bound");
         return FR_ERR_OOM;
     }
-    free_queue(ctx);
-    if (cudaMalloc(&ctx->q_mem, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        ctx->q_mem = nullptr;
-        ctx_error(ctx, "cudaMalloc(%zu) for the queue sweep failed", bytes);
-        return FR_ERR_OOM;
+    // Another cluster size lays the same memory out again where it is large enough: a V-cycle
+    // and the rounds of active scheduling change sizes often, and a cudaFree and cudaMalloc
+    // pair takes longer than a small round.
+    if (!ctx->q_mem || bytes > ctx->q_bytes) {
+        free_queue(ctx);
+        if (cudaMalloc(&ctx->q_mem, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            ctx->q_mem = nullptr;
+            ctx_error(ctx, "cudaMalloc(%zu) for the queue sweep failed", bytes);
+            return FR_ERR_OOM;
+        }
+        ctx->q_bytes = bytes;
     }
-    ctx->q_bytes = bytes;
     ctx->q_ctas = ctas; ctx->q_clusters = cc; ctx->q_n = nn; ctx->q_nnz = mm; ctx->q_k = kk; ctx->q_reps = rr;
     ctx->q_np = pp;
     ctx->q_nu = c.nu; ctx->q_mu = c.mu; ctx->q_vq = c.vq;
@@ -411,4 +419,128 @@ fr_status run_queue_sweep(fr_ctx *ctx, const fr_graph *g, int32_t *part, const B
     }
     *ran = true;
     return FR_OK;
+}
+
+// ------------------------------------------------- one round, one launch ----
+// The pairs of one round (block-disjoint, so none waits for another) through the queue
+// kernel, a cluster for each pair, instead of the sequence boundary scan, step, cluster flow,
+// step.  Those two steps are cooperative launches over the whole grid, some 140 us each for a
+// corridor of a few thousand vertices whatever its size: about forty grid barriers of 2-3 us
+// and dependent loads between them.  A cluster barrier is 0.25 us.
+
+int queue_round_size(fr_ctx *ctx, int P, long long est, double avg_degree, const fr_options *opt) {
+    if (P <= 0 || opt->sweep_sched == 1 || ctx->max_clusters <= 0 || queue_smem() == 0) return -1;
+    const double need = 1.05 * (double)est * (29.0 + 16.0 * avg_degree);
+    const double per_cta = 0.95 * (double)queue_smem();
+    const int force = opt->cluster_ctas ? opt->cluster_ctas : ctx->tune_ctas;
+    constexpr long long kTiny = 512;
+    int best = -1, kept = -1;
+    double bestc = 0, keptc = 0;
+    for (int t = 0; t < fr_ctx::kNumClusterSizes; ++t) {
+        if (ctx->q_cap[t] <= 0) continue;
+        const int c = fr_ctx::kClusterSizes[t];
+        if (force) {
+            if (force == c) return t;
+            continue;
+        }
+        if (need > per_cta * c) continue;
+        // turns of resident clusters times the time of one pair; a corridor of fewer vertices
+        // than one CTA has threads only loses by being spread (122 vertices: 288 us on 4 CTAs,
+        // 308 on 16, the whole call)
+        const double v = est <= kTiny ? (double)c :
+                                        (double)((P + ctx->q_cap[t] - 1) / ctx->q_cap[t]) * kRelTime[t];
+        if (best < 0 || v < bestc) { best = t; bestc = v; }
+        if (ctx->q_mem && ctx->q_ctas == c) { kept = t; keptc = v; }
+    }
+    // the size laid out already, unless another is clearly better
+    return kept >= 0 && keptc <= 1.25 * bestc ? kept : best;
+}
+
+fr_status enqueue_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int k, int P, long long Lmax,
+                              const fr_options *opt, int t, RoundQueue *rq) {
+    *rq = RoundQueue();
+    const int ctas = fr_ctx::kClusterSizes[t];
+    int clusters = std::max(1, std::min(ctx->q_cap[t], P));
+    if (opt->grid_blocks > 0) clusters = std::max(1, std::min(clusters, opt->grid_blocks / ctas));
+    const int reps = opt->mb_reps > 0 ? opt->mb_reps : 1;
+    const fr_status st = ensure_queue(ctx, ctas, clusters, g->n, g->nnz, k, reps, P);
+    if (st == FR_ERR_OOM) return FR_OK;   // no room under the arena bound: the round's own launches
+    if (st != FR_OK) return st;
+    GraphDev *hg = reinterpret_cast<GraphDev *>(ctx->h_stage + kStageRound);
+    static_assert(kStageRound + 64 * sizeof(GraphDev) <= kStageRoundW, "descriptors of every resident cluster");
+    if (clusters > 64) clusters = 64;
+    for (int i = 0; i < clusters; ++i) {
+        GraphDev &gd = hg[i];
+        memset(&gd, 0, sizeof(gd));
+        gd.xadj = g->xadj; gd.adjncy = g->adjncy; gd.adjwgt = g->adjwgt; gd.vwgt = g->vwgt;
+        gd.part = part; gd.dist = ctx->dist; gd.lid = ctx->lid;
+        gd.sob = ctx->q_host[i].sob;
+        gd.blockw = ctx->blockw;
+        gd.n = g->n; gd.nnz = g->nnz; gd.k = k; gd.base = 0; gd.Lmax = Lmax;
+        gd.bl = ctx->bl; gd.blc = ctx->blc; gd.inb = ctx->inb;
+    }
+    CK(cudaMemcpyAsync(ctx->q_graphs, hg, sizeof(GraphDev) * (size_t)clusters, cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaMemsetAsync(ctx->q_prev, 0xFF, sizeof(int) * 2 * (size_t)P, ctx->stream));   // no pair waits
+    // part and the block weights as they are, should a pair outgrow its cluster
+    CK(cudaMemcpyAsync(ctx->spare, part, sizeof(int) * (size_t)g->n, cudaMemcpyDeviceToDevice, ctx->stream));
+    CK(cudaMemcpyAsync(ctx->h_stage + kStageRoundW, ctx->blockw, sizeof(long long) * (size_t)k, cudaMemcpyDeviceToHost,
+                       ctx->stream));
+    QueueArgs q;
+    memset(&q, 0, sizeof(q));
+    q.wt = make_work(ctx, 0, 0, P, g->n, opt);
+    q.wt.vq_cap = (int)ctx->q_vq;
+    q.wt.nu_cap = (int)ctx->q_nu;
+    q.wt.mu_cap = (int)ctx->q_mu;
+    q.wt.crank = ctx->q_crank;
+    q.wt.total_n = g->n;
+    q.slots = ctx->q_slots;
+    q.np = P;
+    q.ticket = ctx->q_ticket;
+    q.prev = ctx->q_prev;
+    q.gabort = ctx->q_gabort;
+    q.wait_ns = kWaitNs;
+    // the ticket and the abort word lie next to each other, and so do the control blocks
+    // and the counters
+    CK(cudaMemsetAsync(ctx->q_ticket, 0, al256(sizeof(int)) + sizeof(int), ctx->stream));
+    CK(cudaMemsetAsync(ctx->q_ctls, 0, al256(sizeof(fr_ctx::QCtl) * (size_t)ctx->q_clusters) +
+                                           4 * sizeof(long long) * (size_t)clusters, ctx->stream));
+    CK(launch_queue_sweep(q, ctas, clusters, ctx->stream));
+    char *h = ctx->h_stage + kStageRoundCtl;
+    CK(cudaMemcpyAsync(h, ctx->q_gabort, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaMemcpyAsync(h + 256, ctx->q_ctls, sizeof(fr_ctx::QCtl) * (size_t)clusters, cudaMemcpyDeviceToHost,
+                       ctx->stream));
+    rq->queued = true;
+    rq->clusters = clusters;
+    return FR_OK;
+}
+
+fr_status finish_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int k, const char *where, RoundQueue *rq) {
+    const char *h = ctx->h_stage + kStageRoundCtl;
+    const int gab = *reinterpret_cast<const int *>(h);
+    const fr_ctx::QCtl *qc = reinterpret_cast<const fr_ctx::QCtl *>(h + 256);
+    memset(&rq->ctl, 0, sizeof(rq->ctl));
+    for (int i = 0; i < rq->clusters; ++i) {
+        const Ctl &c = qc[i].c;
+        rq->ctl.pulses += c.pulses;
+        rq->ctl.relabels += c.relabels;
+        rq->ctl.levels = std::max(rq->ctl.levels, c.levels);
+        rq->ctl.scc_rounds += c.scc_rounds;
+        if (gab != 0 && c.error && !rq->ctl.error) {
+            rq->ctl.error = c.error;
+            rq->ctl.error_where = c.error_where;
+        }
+    }
+    if (gab == 0) return FR_OK;
+    fr_status st = reset_queue_idle(ctx);
+    if (st != FR_OK) return st;
+    if (gab == E_MISFIT) {
+        rq->queued = false;
+        ++ctx->queue_fallbacks;
+        CK(cudaMemcpyAsync(part, ctx->spare, sizeof(int) * (size_t)g->n, cudaMemcpyDeviceToDevice, ctx->stream));
+        CK(cudaMemcpyAsync(ctx->blockw, ctx->h_stage + kStageRoundW, sizeof(long long) * (size_t)k,
+                           cudaMemcpyHostToDevice, ctx->stream));
+        return FR_OK;
+    }
+    if (!rq->ctl.error) rq->ctl.error = gab;
+    return status_from_ctl(ctx, rq->ctl, where);
 }
