@@ -17,14 +17,16 @@
 //
 // GPU form.  Pairs of a round are block-disjoint, so one CTA searches one pair on
 // vertex-indexed state shared by the round.  Each block's queue is an array of gain
-// buckets, each bucket a stack of entries (vertex, version) in global memory with its
-// top in shared memory: a gain change pushes a new entry with the vertex's next version
-// (its stamp is larger than every earlier one, so a stack stays ordered by stamp) and
-// makes the old entry stale; pops skip stale entries.  The initial stacks come from a
-// sort of the boundary by (block, gain, stamp).  One warp runs the moves: the top of
-// each block's highest non-empty bucket (bitmap in shared memory), the TopGain choice,
-// then the moved vertex's arcs 32 at a time -- gain updates, lazy first-touch of a
-// neighbour (its weights to both blocks from its adjacency), and the pushes, placed in
+// buckets, each bucket a stack of entries in global memory with its top in shared
+// memory: a gain change pushes a new entry (its stamp is larger than every earlier one,
+// so a stack stays ordered by stamp) and marks the vertex's old one dead; pops skip dead
+// entries.  The latest entries are in shared memory too, with their vertices' rows, so that
+// most tops are found there: telling a stale top by its vertex's version cost two more
+// dependent loads (with the 12-byte entries it kept, one round of rgg3d 262,144 vertices,
+// k = 64, took 35.5 ms, now 34.0; bound by the chain of dependent loads of the one warp).
+// The initial stacks come from a sort of the boundary by (block, gain, stamp).  One warp
+// runs the moves: the top of each block's highest non-empty bucket (bitmap in shared memory), the TopGain choice,
+// then the moved vertex's arcs 32 at a time -- gain updates and the pushes, placed in
 // arc order so that every bucket stays ordered.  The rollback, the block weights and
 // the boundary candidate list are updated by the whole CTA afterwards.
 #include <climits>
@@ -148,6 +150,8 @@ __device__ __forceinline__ unsigned lanemask_lt() {
 
 constexpr int kFmWords = kFmMaxBuckets / 32;   // bitmap words per block
 
+constexpr int kFmRing = kFmSortSmem;   // latest entries kept where the boundary was sorted (16 bytes each)
+
 struct FmShared {
     int top[2 * kFmMaxBuckets];          // top entry of each (block, bucket) stack, -1 empty
     // where vbits says the top entry is current: its vertex, the entry below it and the
@@ -257,9 +261,8 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
     // 2. initial stacks: entries in sorted order, each below its predecessor in the bucket
     for (int i = threadIdx.x; i < B; i += blockDim.x) {
         const int bk = sr.bk[i];
-        f.ent_v[E + i] = sr.v[i];
-        f.ent_ver[E + i] = 0;
-        f.ent_below[E + i] = (i > 0 && sr.bk[i - 1] == bk) ? (int)(E + i - 1) : -1;
+        f.ent[E + i] = make_int2(sr.v[i], (i > 0 && sr.bk[i - 1] == bk) ? (int)(E + i - 1) : -1);
+        f.cur[sr.v[i]] = (int)(E + i) + 1;
         if (i + 1 == B || sr.bk[i + 1] != bk) {
             S.top[bk] = (int)(E + i);
             S.topv[bk] = sr.v[i];
@@ -270,7 +273,8 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
             atomicOr(&S.vbits[bk >> 5], 1u << (bk & 31));
         }
     }
-    __syncthreads();
+    __syncthreads();   // (the sort's shared memory is free from here: the ring)
+    int4 *ring = reinterpret_cast<int4 *>(fm_smem + sizeof(FmShared));   // {vertex or -1, entry below, row}
 
     mark(T_FM_SORT);
     // 3. the moves (warp 0).  vbits: the top entry of a stack is known to be current
@@ -287,6 +291,8 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
         long long idle = 0;
         long long nxt = E + B;
         const long long eend = f.eoff[p + 1];   // entries of this pair: [E, eend)
+        const long long ring0 = E + B;          // first entry pushed by a move
+        auto in_ring = [&](long long e) { return e >= ring0 && e >= nxt - kFmRing; };
         bool bad = false;
         for (;;) {
             // top of each block: highest bucket whose top entry is current
@@ -307,16 +313,24 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
                     int ok = 0;
                     if (lane == 0) {
                         const int e = S.top[key];
-                        const int v = f.ent_v[e];
-                        const int ev = f.ent_ver[e], below = f.ent_below[e];
-                        const unsigned char fl = f.flags[v];
-                        const int vv = f.ver[v], x0 = __ldg(G.xadj + v), x1 = __ldg(G.xadj + v + 1);
-                        ok = (fl & kFmInQ) && !(fl & kFmMoved) && vv == ev;
+                        int4 t;
+                        if (in_ring(e)) {
+                            t = ring[e & (kFmRing - 1)];
+                        } else {
+                            const int2 h = f.ent[e];
+                            t = make_int4(h.x, h.y, 0, 0);
+                            if (h.x >= 0) {
+                                t.z = __ldg(G.xadj + h.x);
+                                t.w = __ldg(G.xadj + h.x + 1);
+                            }
+                        }
+                        const int below = t.y;
+                        ok = t.x >= 0;
                         if (ok) {
-                            S.topv[key] = v;
+                            S.topv[key] = t.x;
                             S.topb[key] = below;
-                            S.topj0[key] = x0;
-                            S.topj1[key] = x1;
+                            S.topj0[key] = t.z;
+                            S.topj1[key] = t.w;
                             S.vbits[key >> 5] |= 1u << (key & 31);
                         } else {
                             S.top[key] = below;
@@ -350,7 +364,8 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
             const long long cv = __ldg(G.vwgt + v);
             __syncwarp();
             // pop; the check of the entry below starts now (lane 0)
-            int v2 = -1, ev2 = 0, b2 = -1;
+            int v2 = -1, b2 = -1, x20 = 0, x21 = 0;
+            bool row2 = false;   // (its row is known)
             if (lane == 0) {
                 S.top[key] = below;
                 S.vbits[key >> 5] &= ~(1u << (key & 31));
@@ -358,31 +373,37 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
                 f.flags[v] = kFmTouched | kFmMoved;
                 G.part[v] = to;
                 ml[nm] = v;
-                if (below >= 0) { v2 = f.ent_v[below]; ev2 = f.ent_ver[below]; b2 = f.ent_below[below]; }
+                if (below >= 0) {
+                    if (in_ring(below)) {
+                        const int4 t = ring[below & (kFmRing - 1)];
+                        v2 = t.x; b2 = t.y; x20 = t.z; x21 = t.w;
+                        row2 = true;
+                    } else {
+                        const int2 h = f.ent[below];
+                        v2 = h.x; b2 = h.y;
+                    }
+                }
             }
             ++nm;
             cut -= g;
             __syncwarp();
-            unsigned char fl2 = 0;
-            int ver2 = -1, x20 = 0, x21 = 0;
             bool hit2 = false;   // the entry below belongs to a neighbour updated by this move
             // the moved vertex's arcs, 32 at a time in adjacency order
             for (int jb = j0; jb < j1; jb += 32) {
                 const int j = jb + lane;
                 int u = -1, wt = 0;
                 if (j < j1) { u = __ldg(G.adjncy + j); wt = __ldg(G.adjwgt + j); }
-                if (jb == j0 && lane == 0 && below >= 0) {   // second half of the check
-                    fl2 = f.flags[v2]; ver2 = f.ver[v2];
+                if (jb == j0 && v2 >= 0 && !row2) {   // second half of the check (lane 0)
                     x20 = __ldg(G.xadj + v2); x21 = __ldg(G.xadj + v2 + 1);
                 }
                 bool act = false;
-                int nin = 0, nex = 0, ukey = -1, okey = -1, nver = 0, ux0 = 0, ux1 = 0;
+                int nin = 0, nex = 0, ukey = -1, okey = -1, old = 0, ux0 = 0, ux1 = 0;
                 unsigned char fl = 0;
                 if (u >= 0) {
                     // independent loads, issued together
                     const int pu = G.part[u];
                     fl = f.flags[u];
-                    const int in0 = f.in[u], ex0 = f.ext[u], ver0 = f.ver[u];
+                    const int in0 = f.in[u], ex0 = f.ext[u], cur0 = f.cur[u];
                     ux0 = __ldg(G.xadj + u); ux1 = __ldg(G.xadj + u + 1);
                     if ((pu == a || pu == b) && !(fl & kFmMoved)) {
                         act = true;
@@ -391,8 +412,10 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
                         else { nin += wt; nex -= wt; }
                         const int sb = pu == a ? 0 : kFmMaxBuckets;
                         ukey = sb + (nex - nin) + gmax;
-                        if (fl & kFmInQ) okey = sb + (ex0 - in0) + gmax;
-                        nver = ver0 + 1;
+                        if (fl & kFmInQ) {
+                            okey = sb + (ex0 - in0) + gmax;
+                            old = cur0;
+                        }
                     }
                 }
                 const int v2b = __shfl_sync(0xffffffffu, v2, 0);
@@ -402,10 +425,14 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
                 const unsigned fm_ = __ballot_sync(0xffffffffu, fresh);
                 if (fresh) vl[tl + __popc(fm_ & lanemask_lt())] = u;
                 tl += __popc(fm_);
-                // u's old entry is stale now.  If it is the known-current top of its stack,
+                // u's old entry is dead now.  If it is the known-current top of its stack,
                 // take it off: the entry below becomes the top, not yet checked.  (A top known
                 // to be current that belongs to another vertex stays current.)  Done before any
                 // lane reads a top for a push.
+                if (old > 0) {
+                    f.ent[old - 1].x = -1;
+                    if (in_ring(old - 1)) ring[(old - 1) & (kFmRing - 1)].x = -1;
+                }
                 if (okey >= 0 && ((S.vbits[okey >> 5] >> (okey & 31)) & 1u) && S.topv[okey] == u) {
                     const int nb = S.topb[okey];
                     S.top[okey] = nb;
@@ -422,7 +449,7 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
                 }
                 const long long pos = nxt + __popc(pm & lanemask_lt());
                 // lanes pushing onto the same stack: the lower lane's entry goes below
-                const unsigned grp = __match_any_sync(0xffffffffu, push ? ukey : -1 - lane);
+                const unsigned grp = __match_any_sync(0xffffffffu, push ? ukey : -1);   // (its time grows with the distinct values)
                 const unsigned lower = grp & lanemask_lt();
                 const long long pos_lower = __shfl_sync(0xffffffffu, pos, lower ? 31 - __clz(lower) : lane);
                 int ubelow = -1;
@@ -431,12 +458,11 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
                 if (act) {
                     f.in[u] = nin;
                     f.ext[u] = nex;
-                    f.ver[u] = nver;
+                    if (push) f.cur[u] = (int)pos + 1;
                     f.flags[u] = (unsigned char)(kFmTouched | (push ? kFmInQ : 0));
                     if (push) {
-                        f.ent_v[pos] = u;
-                        f.ent_ver[pos] = nver;
-                        f.ent_below[pos] = ubelow;
+                        f.ent[pos] = make_int2(u, ubelow);
+                        ring[pos & (kFmRing - 1)] = make_int4(u, ubelow, ux0, ux1);
                         if ((grp & ~lower & ~(1u << lane)) == 0) {   // highest lane of the group
                             S.top[ukey] = (int)pos;
                             S.topv[ukey] = u;
@@ -454,12 +480,11 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
             if (bad) break;
             if (s == 0) { wA -= cv; wB += cv; } else { wB -= cv; wA += cv; }   // (its load overlapped the arcs)
             // the entry below the popped one: current, and still the top of its stack?
-            if (lane == 0 && below >= 0) {
-                if (j0 >= j1) {   // no arcs: the second half of the check did not run
-                    fl2 = f.flags[v2]; ver2 = f.ver[v2];
+            if (lane == 0 && v2 >= 0) {
+                if (j0 >= j1 && !row2) {   // no arcs: the second half of the check did not run
                     x20 = __ldg(G.xadj + v2); x21 = __ldg(G.xadj + v2 + 1);
                 }
-                if (!hit2 && S.top[key] == below && (fl2 & kFmInQ) && !(fl2 & kFmMoved) && ver2 == ev2) {
+                if (!hit2 && S.top[key] == below) {
                     S.topv[key] = v2;
                     S.topb[key] = b2;
                     S.topj0[key] = x20;
@@ -498,7 +523,7 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
     for (int i = threadIdx.x; i < tl; i += blockDim.x) {
         const int v = vl[i];
         f.flags[v] = 0;
-        f.ver[v] = 0;
+        f.cur[v] = 0;
     }
     // 5. block weights and boundary candidates of the kept moves (the moved vertex and
     // its neighbours in its old block, as the commit of a flow does)

@@ -21,14 +21,14 @@ struct FmRes {
 // are zero between rounds: every search clears what it touched.
 struct FmDev {
     int *in, *ext;              // [n] weight to the vertex's own block / to the pair's other block
-    int *ver;                   // [n] queue version: an entry is current iff its version matches
+    int *cur;                   // [n] the vertex's latest stack entry + 1 (0: none)
     unsigned char *flags;       // [n] kFmTouched | kFmInQ | kFmMoved
     int *vlist;                 // [n] per pair region: boundary vertices, then vertices touched later
     int *mlog;                  // [n] per pair region: vertices moved, in order
     int *blockn, *blockarcs;    // [k] vertex and arc counts of the blocks (zeroed by fm_offsets)
     long long *voff, *eoff;     // [P], [P + 1] region offsets: vertices (vlist, mlog), stack entries
     int *np, *bcnt;             // [P] pair vertex counts, boundary vertices gathered
-    int *ent_v, *ent_ver, *ent_below;   // [ecap] bucket stack entries
+    int2 *ent;                  // [ecap] bucket stack entries: {vertex, or -1 once dead; entry below}
     unsigned long long *skey;   // [scap] sort scratch for boundaries beyond shared memory
     int *sbkt, *sv;             // [scap]
     FmRes *res;                 // [P]
