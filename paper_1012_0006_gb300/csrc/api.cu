@@ -255,7 +255,7 @@ fr_status ensure_fm(fr_ctx *ctx, int n, int nnz, int k, int P) {
     const long long ecap = nn + mm, scap = 2 * nn;
     size_t b = 0;
     auto add = [&](size_t elem, long long cnt) { b += ((elem * (size_t)cnt + 255) / 256) * 256; };
-    add(4, nn); add(4, nn); add(4, nn); add(1, nn);         // in ext cur flags
+    add(16, nn);                                            // rec
     add(4, nn); add(4, nn);                                 // vlist mlog
     add(4, kk); add(4, kk);                                 // blockn blockarcs
     add(8, pp); add(8, pp + 1); add(4, pp); add(4, pp);     // voff eoff np bcnt
@@ -277,8 +277,7 @@ fr_status ensure_fm(fr_ctx *ctx, int n, int nnz, int k, int P) {
     ctx->fm_n = (int)nn; ctx->fm_nnz = (int)mm; ctx->fm_k = kk; ctx->fm_p = pp;
     char *p = reinterpret_cast<char *>(ctx->fm_mem);
     FmDev &f = ctx->fm;
-    f.in = carve<int>(p, nn); f.ext = carve<int>(p, nn); f.cur = carve<int>(p, nn);
-    f.flags = carve<unsigned char>(p, nn);
+    f.rec = carve<int4>(p, nn);
     f.vlist = carve<int>(p, nn); f.mlog = carve<int>(p, nn);
     f.blockn = carve<int>(p, kk); f.blockarcs = carve<int>(p, kk);
     f.voff = carve<long long>(p, pp); f.eoff = carve<long long>(p, pp + 1);
@@ -287,9 +286,7 @@ fr_status ensure_fm(fr_ctx *ctx, int n, int nnz, int k, int P) {
     f.skey = carve<unsigned long long>(p, scap); f.sbkt = carve<int>(p, scap); f.sv = carve<int>(p, scap);
     f.res = carve<FmRes>(p, pp);
     f.ecap = ecap; f.scap = scap;
-    // per-vertex state is zero between searches; block counts start at zero
-    CK(cudaMemsetAsync(f.cur, 0, sizeof(int) * (size_t)nn, ctx->stream));
-    CK(cudaMemsetAsync(f.flags, 0, (size_t)nn, ctx->stream));
+    // block counts start at zero
     CK(cudaMemsetAsync(f.blockn, 0, sizeof(int) * (size_t)kk, ctx->stream));
     CK(cudaMemsetAsync(f.blockarcs, 0, sizeof(int) * (size_t)kk, ctx->stream));
     destroy_graph_cache(ctx);   // captured sweeps hold pointers into the old workspace

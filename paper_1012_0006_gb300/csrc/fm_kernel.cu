@@ -16,19 +16,24 @@
 // go by a seeded bit; the best state is the smallest (overload, cut, max block weight).
 //
 // GPU form.  Pairs of a round are block-disjoint, so one CTA searches one pair on
-// vertex-indexed state shared by the round.  Each block's queue is an array of gain
-// buckets, each bucket a stack of entries in global memory with its top in shared
-// memory: a gain change pushes a new entry (its stamp is larger than every earlier one,
-// so a stack stays ordered by stamp) and marks the vertex's old one dead; pops skip dead
-// entries.  The latest entries are in shared memory too, with their vertices' rows, so that
-// most tops are found there: telling a stale top by its vertex's version cost two more
-// dependent loads (with the 12-byte entries it kept, one round of rgg3d 262,144 vertices,
-// k = 64, took 35.5 ms, now 34.0; bound by the chain of dependent loads of the one warp).
-// The initial stacks come from a sort of the boundary by (block, gain, stamp).  One warp
-// runs the moves: the top of each block's highest non-empty bucket (bitmap in shared memory), the TopGain choice,
-// then the moved vertex's arcs 32 at a time -- gain updates and the pushes, placed in
-// arc order so that every bucket stays ordered.  The rollback, the block weights and
-// the boundary candidate list are updated by the whole CTA afterwards.
+// 16-byte vertex records shared by the round, one load for all that a move needs of a
+// neighbour.  Each block's queue is an array of gain buckets, each bucket a stack of
+// entries in global memory with its top in shared memory: a gain change pushes a new
+// entry (its stamp is larger than every earlier one, so a stack stays ordered by stamp)
+// and marks the vertex's old one dead; pops skip dead entries.  The latest 4,096 entries
+// are in shared memory too, with their vertices' rows, so that most tops are found there.
+// The initial stacks come from a sort of the boundary by (block, gain, stamp).
+// One warp runs the moves: the top of each block's highest non-empty bucket (16 lanes a
+// block look at 16 buckets; flags tell which groups of 16 may hold an entry), the TopGain
+// choice, then the moved vertex's arcs 32 at a time -- gain updates and the pushes, placed
+// in arc order so that every bucket stays ordered.  The other warps read the rows of the
+// entries that are pushed, and the records of the rows' neighbours, into L1 before they are
+// popped.  The kept moves, the block weights and the boundary candidate list are written by
+// the whole CTA afterwards.  Bound by the one warp's chain, about 2,100 cycles a move (shared
+// memory and L1 round trips, and five cycles an instruction).  One round of rgg3d 262,144
+// vertices, k = 64 with its flows: 35.5 ms with separate arrays, entries told stale by the
+// vertex's version and a lookahead of one entry; 32.1 with dead entries and the ring; 25.0
+// with records, the warps that read ahead (2.1 ms of it) and the search by groups.
 #include <climits>
 
 #include "fm_kernel.cuh"
@@ -82,30 +87,32 @@ __global__ void __launch_bounds__(1024) fm_offsets_kernel(Work w, FmDev f) {
     for (int i = threadIdx.x; i < G.k; i += blockDim.x) f.blockn[i] = f.blockarcs[i] = 0;
 }
 
-// Weights of every paired vertex to its own block and to the partner block within
-// G[A u B] (so that the moves never scan an adjacency for them); vertices with an edge
-// to the partner are the boundary and enter their pair's list.
+// The records of all vertices: the weights of a paired vertex to its own block and to the
+// partner block within G[A u B] (so that the moves never scan an adjacency for them) and
+// its row; vertices with an edge to the partner are the boundary and enter their pair's list.
 __global__ void __launch_bounds__(kFmTPB) fm_gather_kernel(Work w, FmDev f) {
     if ((w.prev_err && __ldcg(w.prev_err)) || __ldcg(&w.ctl->error)) return;
     const GraphDev G = w.graphs[0];
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < G.n; v += gridDim.x * blockDim.x) {
         const int b = G.part[v];
         const int s = side_of(G, b);
-        if (s < 0) continue;
+        if (s < 0) {
+            f.rec[v].z = -1;
+            continue;
+        }
         const PairDev P = w.pairs[s >> 1];
         const int partner = (s & 1) ? P.a : P.b;
         int in = 0, ex = 0;
-        const int j1 = __ldg(G.xadj + v + 1);
-        for (int j = __ldg(G.xadj + v); j < j1; ++j) {
+        const int j0 = __ldg(G.xadj + v), j1 = __ldg(G.xadj + v + 1);
+        for (int j = j0; j < j1; ++j) {
             const int pu = G.part[__ldg(G.adjncy + j)];
             const int wt = __ldg(G.adjwgt + j);
             if (pu == b) in += wt;
             else if (pu == partner) ex += wt;
         }
-        f.in[v] = in;
-        f.ext[v] = ex;
+        // (a weight beyond ten bits ends the search before it reads the record)
+        f.rec[v] = make_int4((in & 1023) | (ex & 1023) << 10 | (int)((unsigned)(j1 - j0) << 20), 0, b, j0);
         if (ex == 0) continue;
-        f.flags[v] = kFmTouched | kFmInQ;
         const int pos = atomicAdd(f.bcnt + (s >> 1), 1);
         f.vlist[f.voff[s >> 1] + pos] = v;
     }
@@ -148,22 +155,64 @@ __device__ __forceinline__ unsigned lanemask_lt() {
     return m;
 }
 
-constexpr int kFmWords = kFmMaxBuckets / 32;   // bitmap words per block
+constexpr int kFmGroup = 16, kFmGroups = kFmMaxBuckets / kFmGroup;   // buckets of a group, groups of a block
 
+constexpr int kFmAhead = kFmTPB / 32 - 1;   // warps that read ahead of the moves
+constexpr int kFmFresh = 64;                // pushed entries older than this are left
+constexpr int kFmSeedsAhead = 16;           // entries of each block's start they are ahead
+constexpr int kFmIdle = 1 << 22;            // polls without work before such a warp gives up
 constexpr int kFmRing = kFmSortSmem;   // latest entries kept where the boundary was sorted (16 bytes each)
 
-struct FmShared {
+struct __align__(16) FmShared {
     int top[2 * kFmMaxBuckets];          // top entry of each (block, bucket) stack, -1 empty
-    // where vbits says the top entry is current: its vertex, the entry below it and the
-    // vertex's adjacency range (so a move reads no entry and no offsets from memory)
-    int topv[2 * kFmMaxBuckets], topb[2 * kFmMaxBuckets];
-    int topj0[2 * kFmMaxBuckets], topj1[2 * kFmMaxBuckets];
-    unsigned bits[2 * kFmWords];         // non-empty stacks (possibly holding only stale entries)
-    unsigned vbits[2 * kFmWords];        // the top entry is known to be current
+    unsigned char group[2 * kFmGroups];  // groups of stacks that may hold an entry
     long long red[kFmTPB / 32];
     int best_len, tried;
+    int pushes, moves, done;             // progress, for the warps that read ahead
+    unsigned sink;                       // (their loads end here)
     long long best_cut, best_wA, best_wB;
 };
+
+// What the warps behind the moving one do: they read the rows, and the records of the rows'
+// neighbours, that it will need next into L1, so that a move finds them there.  The start's
+// entries come first, from the top of each block down and two a move; then the pushed
+// entries, while they are new.
+__device__ __forceinline__ void fm_ahead(const GraphDev &G, const FmDev &f, FmShared &S, const int4 *ring,
+                                         long long E, int n0, int B) {
+    const int lane = threadIdx.x & 31, me = (threadIdx.x >> 5) - 1;
+    const int nnz = __ldg(G.xadj + G.n);
+    unsigned acc = 0;
+    auto warm = [&](int v, int j0, int j1) {
+        acc ^= (unsigned)__ldg(G.vwgt + v);
+        for (int j = j0 + lane; j < min(j1, nnz); j += 32)
+            acc ^= (unsigned)__ldg(G.adjwgt + j) ^ (unsigned)f.rec[__ldg(G.adjncy + j)].x;
+    };
+    int seed = me, push = me;
+    for (int polls = 0; polls < kFmIdle; ++polls) {
+        if (*(volatile int *)&S.done) break;
+        const int pushes = *(volatile int *)&S.pushes, moves = *(volatile int *)&S.moves;
+        if (push < pushes) {
+            if (push < pushes - kFmFresh) push += (pushes - kFmFresh - push + kFmAhead - 1) / kFmAhead * kFmAhead;
+            if (push >= pushes) continue;
+            const int4 t = ring[(int)((E + B + push) & (kFmRing - 1))];
+            push += kFmAhead;
+            if (t.x >= 0) warm(t.x, t.z, t.w);
+            polls = 0;
+        } else if (seed < 2 * max(n0, B - n0) && seed < 2 * (moves + kFmSeedsAhead)) {
+            const int lo = (seed & 1) ? n0 : 0, i = ((seed & 1) ? B : n0) - 1 - (seed >> 1);
+            seed += kFmAhead;
+            const int v = i >= lo ? f.ent[E + i].x : -1;
+            if (v >= 0) {
+                const int4 r = f.rec[v];
+                warm(v, r.w, r.w + fm_deg(r.x));
+            }
+            polls = 0;
+        } else {
+            __nanosleep(100);
+        }
+    }
+    if (acc == 0x9e3779b9u) S.sink = acc;
+}
 
 __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
     extern __shared__ __align__(16) char fm_smem[];
@@ -173,28 +222,18 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
     const PairDev P = w.pairs[p];
     const int a = P.a, b = P.b;
     const int n_p = f.np[p];
-    // the gather ran only without an earlier error; what it marked is cleared on every exit
-    const bool gathered = !(w.prev_err && __ldcg(w.prev_err));
-    const int B = gathered ? f.bcnt[p] : 0;
+    if ((w.prev_err && __ldcg(w.prev_err)) || __ldcg(&w.ctl->error)) return;   // (the gather may not have run)
+    const int B = f.bcnt[p];
     int *vl = f.vlist + f.voff[p];
     int *ml = f.mlog + f.voff[p];
-    auto bail = [&]() {
-        for (int i = threadIdx.x; i < B; i += blockDim.x) f.flags[vl[i]] = 0;
-    };
-    if (!gathered || __ldcg(&w.ctl->error)) {
-        bail();
-        return;
-    }
     FmRes *R = f.res + p;
     const long long wA0 = G.blockw[a], wB0 = G.blockw[b];
     if (n_p == 0 || f.permille <= 0) {
-        bail();
         if (threadIdx.x == 0) *R = FmRes{0, wA0, wB0, 0, wA0, wB0, 0, 0};
         return;
     }
     const int gmax = __ldcg(f.maxwdeg);   // |gain| <= max weighted degree
     if (2 * gmax + 1 > kFmMaxBuckets) {
-        bail();
         if (threadIdx.x == 0) fail(w.ctl, E_TOO_LARGE, 701);
         return;
     }
@@ -226,7 +265,6 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
             if (mq > kFmSortSmem) so += mq;
         }
         if (so + m > f.scap) {
-            bail();
             if (threadIdx.x == 0) fail(w.ctl, E_INTERNAL, 702);
             return;
         }
@@ -238,12 +276,13 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
     for (int i = threadIdx.x; i < m; i += blockDim.x) {
         if (i < B) {
             const int v = vl[i];
-            const int side = G.part[v] == a ? 0 : 1;
-            const int g = f.ext[v] - f.in[v];
+            const int4 r = f.rec[v];
+            const int side = r.z == a ? 0 : 1;
+            const int g = fm_ext(r.x) - fm_in(r.x);
             sr.bk[i] = side * kFmMaxBuckets + g + gmax;
             sr.st[i] = splitmix64(fs ^ (unsigned long long)(unsigned)v) >> 1;
             sr.v[i] = v;
-            if (side == 0) c0 += f.ext[v];
+            if (side == 0) c0 += fm_ext(r.x);
         } else {
             sr.bk[i] = INT_MAX;
             sr.st[i] = ~0ull;
@@ -251,7 +290,7 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
         }
     }
     for (int i = threadIdx.x; i < 2 * kFmMaxBuckets; i += blockDim.x) S.top[i] = -1;
-    for (int i = threadIdx.x; i < 2 * kFmWords; i += blockDim.x) S.bits[i] = S.vbits[i] = 0;
+    for (int i = threadIdx.x; i < 2 * kFmGroups; i += blockDim.x) S.group[i] = 0;
     for (int o = 16; o > 0; o >>= 1) c0 += __shfl_down_sync(0xffffffffu, c0, o);
     if (lane == 0) S.red[warp] = c0;
     __syncthreads();
@@ -260,186 +299,146 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
     for (int i = 0; i < kFmTPB / 32; ++i) cut0 += S.red[i];
     // 2. initial stacks: entries in sorted order, each below its predecessor in the bucket
     for (int i = threadIdx.x; i < B; i += blockDim.x) {
-        const int bk = sr.bk[i];
-        f.ent[E + i] = make_int2(sr.v[i], (i > 0 && sr.bk[i - 1] == bk) ? (int)(E + i - 1) : -1);
-        f.cur[sr.v[i]] = (int)(E + i) + 1;
+        const int bk = sr.bk[i], v = sr.v[i];
+        const int below = (i > 0 && sr.bk[i - 1] == bk) ? (int)(E + i - 1) : -1;
+        f.ent[E + i] = make_int2(v, below);
+        f.rec[v].y = (int)(E + i) + 1;
         if (i + 1 == B || sr.bk[i + 1] != bk) {
             S.top[bk] = (int)(E + i);
-            S.topv[bk] = sr.v[i];
-            S.topb[bk] = (i > 0 && sr.bk[i - 1] == bk) ? (int)(E + i - 1) : -1;
-            S.topj0[bk] = __ldg(G.xadj + sr.v[i]);
-            S.topj1[bk] = __ldg(G.xadj + sr.v[i] + 1);
-            atomicOr(&S.bits[bk >> 5], 1u << (bk & 31));
-            atomicOr(&S.vbits[bk >> 5], 1u << (bk & 31));
+            S.group[bk / kFmGroup] = 1;
         }
     }
+    int n0 = 0;   // boundary vertices of block a: the first n0 entries
+    for (int h = B; n0 < h;) {
+        const int mid = (n0 + h) >> 1;
+        if (sr.bk[mid] < kFmMaxBuckets) n0 = mid + 1;
+        else h = mid;
+    }
+    if (threadIdx.x == 0) S.pushes = S.moves = S.done = 0;
     __syncthreads();   // (the sort's shared memory is free from here: the ring)
     int4 *ring = reinterpret_cast<int4 *>(fm_smem + sizeof(FmShared));   // {vertex or -1, entry below, row}
+    for (int i = threadIdx.x; i < kFmRing; i += blockDim.x) ring[i] = make_int4(-1, -1, 0, 0);
+    __syncthreads();
 
     mark(T_FM_SORT);
-    // 3. the moves (warp 0).  vbits: the top entry of a stack is known to be current
-    // (set by a push or a check, cleared when the top is popped or goes stale), with its
-    // vertex, the entry below and the adjacency range cached.  While
-    // a move updates its neighbours, lane 0 checks the entry below the popped one, so
-    // that the next pop from the same stack usually needs no memory round trip.
-    if (warp == 0) {
+    // 3. the moves (warp 0)
+    if (warp > 0) {
+        fm_ahead(G, f, S, ring, E, n0, B);
+    } else {
         const long long Lmax = G.Lmax;
-        const long long limit = (long long)f.permille * n_p / 1000;
+        const int limit = (int)min((long long)f.permille * n_p / 1000, (long long)INT_MAX - 1);
         long long cut = cut0, wA = wA0, wB = wB0;
         long long bcut = cut, bwA = wA, bwB = wB;
-        int nm = 0, best_len = 0, tl = B;   // tl: end of the touched list in vl
-        long long idle = 0;
-        long long nxt = E + B;
-        const long long eend = f.eoff[p + 1];   // entries of this pair: [E, eend)
-        const long long ring0 = E + B;          // first entry pushed by a move
-        auto in_ring = [&](long long e) { return e >= ring0 && e >= nxt - kFmRing; };
+        long long bmx = wA > wB ? wA : wB, bov = bmx > Lmax ? bmx - Lmax : 0;
+        int nm = 0, best_len = 0;
+        int idle = 0;
+        int nxt = (int)E + B;
+        const int eend = (int)f.eoff[p + 1];   // entries of this pair: [E, eend)
+        const int ring0 = nxt;                 // first entry pushed by a move
+        unsigned ties = 0;                     // bits of moves nm & ~31 on
+        bool over = bov > 0;                   // a block is overloaded
+        const int hl = lane & 15, side = lane >> 4;
+        int hg0 = kFmGroups - 1, hg1 = kFmGroups - 1;   // no group above these holds an entry
         bool bad = false;
         for (;;) {
-            // top of each block: highest bucket whose top entry is current
-            int tb[2];
-            for (int s = 0; s < 2; ++s) {
-                tb[s] = -1;
-                for (;;) {
-                    int best = -1;   // lane L looks at the words 2L, 2L + 1, from the top
-                    for (int k2 = 1; k2 >= 0; --k2) {
-                        const unsigned word = S.bits[s * kFmWords + lane * 2 + k2];
-                        if (best < 0 && word) best = (lane * 2 + k2) * 32 + 31 - __clz(word);
-                    }
-                    const unsigned has = __ballot_sync(0xffffffffu, best >= 0);
-                    if (!has) break;
-                    const int hb = __shfl_sync(0xffffffffu, best, 31 - __clz(has));
-                    const int key = s * kFmMaxBuckets + hb;
-                    if ((S.vbits[key >> 5] >> (key & 31)) & 1u) { tb[s] = hb; break; }
-                    int ok = 0;
-                    if (lane == 0) {
-                        const int e = S.top[key];
-                        int4 t;
-                        if (in_ring(e)) {
+            // top of each block: the highest bucket with a live entry (lanes 0 to 15 look at
+            // the buckets of block a's highest group, 16 to 31 at those of block b's); dead
+            // entries above it go
+            int tb[2], hb;
+            int4 t;
+            const int ring_lo = max(ring0, nxt - kFmRing);   // entries from here on are in the ring
+            int hg = lane < 16 ? hg0 : hg1, key0 = side * kFmMaxBuckets + hg * kFmGroup;
+            int mine = hg >= 0 ? S.top[key0 + hl] : -1;      // this lane's stack
+            for (;;) {
+                const unsigned has = (__ballot_sync(0xffffffffu, mine >= 0) >> (lane & 16)) & 0xffffu;
+                const int w16 = has ? 31 - __clz(has) : 0;
+                int e = __shfl_sync(0xffffffffu, mine, (lane & 16) + w16);
+                hb = has ? hg * kFmGroup + w16 : -1;
+                t = make_int4(-1, -1, 0, 0);
+                if (e >= ring_lo) t = ring[e & (kFmRing - 1)];
+                if (!__any_sync(0xffffffffu, hg >= 0 && t.x < 0)) break;
+                if (e >= 0 && t.x < 0) {   // an entry from before the ring, or a dead one (uniform within a half)
+                    const bool dead = e >= ring_lo;
+                    if (dead) e = t.y;
+                    while (e >= 0) {
+                        if (e >= ring_lo) {
                             t = ring[e & (kFmRing - 1)];
                         } else {
                             const int2 h = f.ent[e];
                             t = make_int4(h.x, h.y, 0, 0);
                             if (h.x >= 0) {
-                                t.z = __ldg(G.xadj + h.x);
-                                t.w = __ldg(G.xadj + h.x + 1);
+                                const int4 r = f.rec[h.x];
+                                t.z = r.w;
+                                t.w = r.w + fm_deg(r.x);
                             }
                         }
-                        const int below = t.y;
-                        ok = t.x >= 0;
-                        if (ok) {
-                            S.topv[key] = t.x;
-                            S.topb[key] = below;
-                            S.topj0[key] = t.z;
-                            S.topj1[key] = t.w;
-                            S.vbits[key >> 5] |= 1u << (key & 31);
-                        } else {
-                            S.top[key] = below;
-                            if (below < 0) S.bits[key >> 5] &= ~(1u << (key & 31));
-                        }
+                        if (t.x >= 0) break;
+                        e = t.y;
                     }
-                    ok = __shfl_sync(0xffffffffu, ok, 0);
+                    if (hl == w16 && e != mine) S.top[key0 + hl] = mine = e;
+                }
+                if (__any_sync(0xffffffffu, hg >= 0 && !has)) {   // a group without entries: the next one
+                    if (hg >= 0 && !has && hl == 0) S.group[side * kFmGroups + hg] = 0;
                     __syncwarp();
-                    if (ok) { tb[s] = hb; break; }
+                    const uint2 fl = reinterpret_cast<const uint2 *>(S.group)[lane];
+                    const int g8 = fl.y ? 7 - (__clz(fl.y) >> 3) : 3 - (__clz(fl.x) >> 3);
+                    const int g = fl.x | fl.y ? hl * 8 + g8 : -1;
+                    hg0 = __reduce_max_sync(0xffffffffu, lane < 16 ? g : -1);
+                    hg1 = __reduce_max_sync(0xffffffffu, lane < 16 ? -1 : g);
+                    hg = lane < 16 ? hg0 : hg1;
+                    key0 = side * kFmMaxBuckets + hg * kFmGroup;
+                    mine = hg >= 0 ? S.top[key0 + hl] : -1;
+                } else if (!__any_sync(0xffffffffu, has && t.x < 0)) {
+                    break;
                 }
             }
+            tb[0] = __shfl_sync(0xffffffffu, hb, 0);
+            tb[1] = __shfl_sync(0xffffffffu, hb, 16);
             if (tb[0] < 0 && tb[1] < 0) break;
-            int s;
-            if (wA > Lmax || wB > Lmax) {
+            if ((nm & 31) == 0) ties = __ballot_sync(0xffffffffu, splitmix64(~fs ^ (unsigned long long)(nm + lane)) & 1);
+            int s = tb[0] == tb[1] ? (int)(ties >> (nm & 31)) & 1 : tb[0] < tb[1];
+            if (over) {
                 s = wA >= wB ? 0 : 1;
-                if (tb[s] < 0) s = 1 - s;
-            } else if (tb[0] < 0) {
-                s = 1;
-            } else if (tb[1] < 0) {
-                s = 0;
-            } else if (tb[0] != tb[1]) {
-                s = tb[0] > tb[1] ? 0 : 1;
-            } else {
-                s = (int)(splitmix64(~fs ^ (unsigned long long)nm) & 1);
+                if ((s ? tb[1] : tb[0]) < 0) s = 1 - s;
             }
-            const int key = s * kFmMaxBuckets + tb[s];
-            const int v = S.topv[key], below = S.topb[key];
-            const int j0 = S.topj0[key], j1 = S.topj1[key];
-            const int g = tb[s] - gmax;
-            const int from = s ? b : a, to = s ? a : b;
+            const int ts = s ? tb[1] : tb[0], key = s * kFmMaxBuckets + ts;
+            const int v = __shfl_sync(0xffffffffu, t.x, s * 16), j0 = __shfl_sync(0xffffffffu, t.z, s * 16);
+            const int j1 = __shfl_sync(0xffffffffu, t.w, s * 16);
+            const int g = ts - gmax;
+            const int from = s ? b : a;
             const long long cv = __ldg(G.vwgt + v);
-            __syncwarp();
-            // pop; the check of the entry below starts now (lane 0)
-            int v2 = -1, b2 = -1, x20 = 0, x21 = 0;
-            bool row2 = false;   // (its row is known)
-            if (lane == 0) {
-                S.top[key] = below;
-                S.vbits[key >> 5] &= ~(1u << (key & 31));
-                if (below < 0) S.bits[key >> 5] &= ~(1u << (key & 31));
-                f.flags[v] = kFmTouched | kFmMoved;
-                G.part[v] = to;
+            // pop
+            if (lane == s * 16) {
+                S.top[key] = t.y;
+                f.rec[v].z = -1;
                 ml[nm] = v;
-                if (below >= 0) {
-                    if (in_ring(below)) {
-                        const int4 t = ring[below & (kFmRing - 1)];
-                        v2 = t.x; b2 = t.y; x20 = t.z; x21 = t.w;
-                        row2 = true;
-                    } else {
-                        const int2 h = f.ent[below];
-                        v2 = h.x; b2 = h.y;
-                    }
-                }
             }
             ++nm;
             cut -= g;
             __syncwarp();
-            bool hit2 = false;   // the entry below belongs to a neighbour updated by this move
             // the moved vertex's arcs, 32 at a time in adjacency order
             for (int jb = j0; jb < j1; jb += 32) {
                 const int j = jb + lane;
                 int u = -1, wt = 0;
                 if (j < j1) { u = __ldg(G.adjncy + j); wt = __ldg(G.adjwgt + j); }
-                if (jb == j0 && v2 >= 0 && !row2) {   // second half of the check (lane 0)
-                    x20 = __ldg(G.xadj + v2); x21 = __ldg(G.xadj + v2 + 1);
-                }
                 bool act = false;
-                int nin = 0, nex = 0, ukey = -1, okey = -1, old = 0, ux0 = 0, ux1 = 0;
-                unsigned char fl = 0;
+                int nex = 0, ukey = -1, old = 0;
+                int4 r = make_int4(0, 0, -1, 0);
                 if (u >= 0) {
-                    // independent loads, issued together
-                    const int pu = G.part[u];
-                    fl = f.flags[u];
-                    const int in0 = f.in[u], ex0 = f.ext[u], cur0 = f.cur[u];
-                    ux0 = __ldg(G.xadj + u); ux1 = __ldg(G.xadj + u + 1);
-                    if ((pu == a || pu == b) && !(fl & kFmMoved)) {
-                        act = true;
-                        nin = in0; nex = ex0;
-                        if (pu == from) { nin -= wt; nex += wt; }
-                        else { nin += wt; nex -= wt; }
-                        const int sb = pu == a ? 0 : kFmMaxBuckets;
-                        ukey = sb + (nex - nin) + gmax;
-                        if (fl & kFmInQ) {
-                            okey = sb + (ex0 - in0) + gmax;
-                            old = cur0;
-                        }
+                    r = f.rec[u];
+                    act = r.z == a || r.z == b;
+                    if (act) {
+                        const int gk = (r.z == a ? 0 : kFmMaxBuckets) + gmax;
+                        old = r.y;
+                        r.x += r.z == from ? wt * 1023 : -wt * 1023;   // wt from in to ext, or back
+                        nex = fm_ext(r.x);
+                        ukey = gk + nex - fm_in(r.x);
                     }
                 }
-                const int v2b = __shfl_sync(0xffffffffu, v2, 0);
-                hit2 |= __ballot_sync(0xffffffffu, act && u == v2b) != 0;
-                // first changes join the touched list (for the cleanup)
-                const bool fresh = act && !(fl & kFmTouched);
-                const unsigned fm_ = __ballot_sync(0xffffffffu, fresh);
-                if (fresh) vl[tl + __popc(fm_ & lanemask_lt())] = u;
-                tl += __popc(fm_);
-                // u's old entry is dead now.  If it is the known-current top of its stack,
-                // take it off: the entry below becomes the top, not yet checked.  (A top known
-                // to be current that belongs to another vertex stays current.)  Done before any
-                // lane reads a top for a push.
-                if (old > 0) {
+                if (old > 0) {   // u's old entry is dead now
                     f.ent[old - 1].x = -1;
-                    if (in_ring(old - 1)) ring[(old - 1) & (kFmRing - 1)].x = -1;
+                    if (old > max(ring0, nxt - kFmRing)) ring[(old - 1) & (kFmRing - 1)].x = -1;
                 }
-                if (okey >= 0 && ((S.vbits[okey >> 5] >> (okey & 31)) & 1u) && S.topv[okey] == u) {
-                    const int nb = S.topb[okey];
-                    S.top[okey] = nb;
-                    if (nb < 0) atomicAnd(&S.bits[okey >> 5], ~(1u << (okey & 31)));
-                    atomicAnd(&S.vbits[okey >> 5], ~(1u << (okey & 31)));
-                }
-                __syncwarp();
                 const bool push = act && nex > 0;
                 const unsigned pm = __ballot_sync(0xffffffffu, push);
                 if (nxt + __popc(pm) > eend) {   // cannot happen: pushes <= boundary + arcs
@@ -447,57 +446,39 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
                     bad = true;
                     break;
                 }
-                const long long pos = nxt + __popc(pm & lanemask_lt());
+                const int pos = nxt + __popc(pm & lanemask_lt());
                 // lanes pushing onto the same stack: the lower lane's entry goes below
                 const unsigned grp = __match_any_sync(0xffffffffu, push ? ukey : -1);   // (its time grows with the distinct values)
                 const unsigned lower = grp & lanemask_lt();
-                const long long pos_lower = __shfl_sync(0xffffffffu, pos, lower ? 31 - __clz(lower) : lane);
+                const int pos_lower = __shfl_sync(0xffffffffu, pos, lower ? 31 - __clz(lower) : lane);
                 int ubelow = -1;
-                if (push) ubelow = lower ? (int)pos_lower : S.top[ukey];
+                if (push) ubelow = lower ? pos_lower : S.top[ukey];
                 __syncwarp();
                 if (act) {
-                    f.in[u] = nin;
-                    f.ext[u] = nex;
-                    if (push) f.cur[u] = (int)pos + 1;
-                    f.flags[u] = (unsigned char)(kFmTouched | (push ? kFmInQ : 0));
+                    *reinterpret_cast<int2 *>(f.rec + u) = make_int2(r.x, push ? pos + 1 : 0);
                     if (push) {
                         f.ent[pos] = make_int2(u, ubelow);
-                        ring[pos & (kFmRing - 1)] = make_int4(u, ubelow, ux0, ux1);
+                        ring[pos & (kFmRing - 1)] = make_int4(u, ubelow, r.w, r.w + fm_deg(r.x));
                         if ((grp & ~lower & ~(1u << lane)) == 0) {   // highest lane of the group
-                            S.top[ukey] = (int)pos;
-                            S.topv[ukey] = u;
-                            S.topb[ukey] = ubelow;
-                            S.topj0[ukey] = ux0;
-                            S.topj1[ukey] = ux1;
-                            atomicOr(&S.bits[ukey >> 5], 1u << (ukey & 31));
-                            atomicOr(&S.vbits[ukey >> 5], 1u << (ukey & 31));
+                            S.top[ukey] = pos;
+                            S.group[ukey / kFmGroup] = 1;
                         }
                     }
                 }
                 nxt += __popc(pm);
+                hg0 = max(hg0, __reduce_max_sync(0xffffffffu, push && ukey < kFmMaxBuckets ? ukey / kFmGroup : -1));
+                hg1 = max(hg1, __reduce_max_sync(0xffffffffu, push ? ukey / kFmGroup - kFmGroups : -1));
                 __syncwarp();
+                if (lane == 0) *(volatile int *)&S.pushes = nxt - ring0;
             }
             if (bad) break;
+            if (lane == 0) *(volatile int *)&S.moves = nm;
             if (s == 0) { wA -= cv; wB += cv; } else { wB -= cv; wA += cv; }   // (its load overlapped the arcs)
-            // the entry below the popped one: current, and still the top of its stack?
-            if (lane == 0 && v2 >= 0) {
-                if (j0 >= j1 && !row2) {   // no arcs: the second half of the check did not run
-                    x20 = __ldg(G.xadj + v2); x21 = __ldg(G.xadj + v2 + 1);
-                }
-                if (!hit2 && S.top[key] == below) {
-                    S.topv[key] = v2;
-                    S.topb[key] = b2;
-                    S.topj0[key] = x20;
-                    S.topj1[key] = x21;
-                    S.vbits[key >> 5] |= 1u << (key & 31);
-                }
-            }
-            __syncwarp();
             // best state: smallest (overload, cut, max block weight)
-            const long long mx = wA > wB ? wA : wB, bmx = bwA > bwB ? bwA : bwB;
-            const long long ov = mx > Lmax ? mx - Lmax : 0, bov = bmx > Lmax ? bmx - Lmax : 0;
+            const long long mx = wA > wB ? wA : wB, ov = mx > Lmax ? mx - Lmax : 0;
+            over = ov > 0;
             if (ov < bov || (ov == bov && (cut < bcut || (cut == bcut && mx < bmx)))) {
-                bcut = cut; bwA = wA; bwB = wB; best_len = nm; idle = 0;
+                bcut = cut; bwA = wA; bwB = wB; bov = ov; bmx = mx; best_len = nm; idle = 0;
             } else if (++idle > limit) {
                 break;
             }
@@ -508,23 +489,18 @@ __global__ void __launch_bounds__(kFmTPB, 1) fm_pair_kernel(Work w, FmDev f) {
             S.best_cut = bcut;
             S.best_wA = bwA;
             S.best_wB = bwB;
-            S.red[0] = tl;
+            *(volatile int *)&S.done = 1;
         }
     }
     __syncthreads();
     mark(T_FM_MOVES);
-    const int best_len = S.best_len, nm = S.tried, tl = (int)S.red[0];
-    // 4. roll back the moves after the best prefix; clear what the search touched
-    for (int i = best_len + threadIdx.x; i < nm; i += blockDim.x) {
+    const int best_len = S.best_len, nm = S.tried;
+    // 4. the moves up to the best prefix
+    for (int i = threadIdx.x; i < best_len; i += blockDim.x) {
         const int v = ml[i];
         G.part[v] = G.part[v] == a ? b : a;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < tl; i += blockDim.x) {
-        const int v = vl[i];
-        f.flags[v] = 0;
-        f.cur[v] = 0;
-    }
     // 5. block weights and boundary candidates of the kept moves (the moved vertex and
     // its neighbours in its old block, as the commit of a flow does)
     if (threadIdx.x == 0) {

@@ -17,13 +17,13 @@ struct FmRes {
     int kept, tried;            // moves kept / made
 };
 
-// Device state of the FM searches of one round (pairs of one graph).  Per-vertex arrays
-// are zero between rounds: every search clears what it touched.
+// Device state of the FM searches of one round (pairs of one graph).
 struct FmDev {
-    int *in, *ext;              // [n] weight to the vertex's own block / to the pair's other block
-    int *cur;                   // [n] the vertex's latest stack entry + 1 (0: none)
-    unsigned char *flags;       // [n] kFmTouched | kFmInQ | kFmMoved
-    int *vlist;                 // [n] per pair region: boundary vertices, then vertices touched later
+    // [n] vertex records, written by every round's gather: {weight to the own block | weight
+    // to the pair's other block << 10 | degree << 20, latest stack entry + 1 (0: not queued),
+    // block (-1: not in a pair of the round, or moved), row begin}
+    int4 *rec;
+    int *vlist;                 // [n] per pair region: boundary vertices
     int *mlog;                  // [n] per pair region: vertices moved, in order
     int *blockn, *blockarcs;    // [k] vertex and arc counts of the blocks (zeroed by fm_offsets)
     long long *voff, *eoff;     // [P], [P + 1] region offsets: vertices (vlist, mlog), stack entries
@@ -37,7 +37,10 @@ struct FmDev {
     int permille;
 };
 
-constexpr unsigned char kFmTouched = 1, kFmInQ = 2, kFmMoved = 4;
+// Ten bits each in a record: |gain| <= weighted degree < 1024, and arc weights are at least 1.
+__host__ __device__ constexpr int fm_in(int x) { return x & 1023; }
+__host__ __device__ constexpr int fm_ext(int x) { return (x >> 10) & 1023; }
+__host__ __device__ constexpr int fm_deg(int x) { return (x >> 20) & 1023; }
 
 // Enqueues the FM searches of the round described by w (one graph with k blocks,
 // w.npairs pairs): block counts, pair regions, boundary gather, one CTA per pair.
