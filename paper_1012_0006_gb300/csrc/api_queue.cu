@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <vector>
 
@@ -22,6 +23,18 @@ namespace {
 // relative time of one pair on clusters of 4, 6, 8, 12, 16 CTAs (measured on 3D rgg and
 // grid pairs; the same table as the round-by-round cluster launches)
 constexpr double kRelTime[fr_ctx::kNumClusterSizes] = {1.25, 1.05, 1.0, 0.85, 0.74};
+// The time of a sweep on clusters of one size: a vertex of the quotient graph is in up to nr
+// pairs that wait for one another, and the clusters have turns = pairs / clusters to take;
+// sqrt(nr^2 + turns^2) times the time of one pair fits both ends.  Corridors of fewer
+// vertices than a cluster of 8 has threads gain little from more CTAs, of fewer than one CTA
+// has none.  Taking the most pairs in flight over a pair's time alone (the chain left out)
+// chose 4 CTAs for rgg3d 524,287 vertices, k = 32 (18 rounds, 155 pairs, 1,316 vertices):
+// 8.2 ms, against 7.5 on 6 and 7.4 on 8; 8 for rgg2d 20,011, k = 7 (346 vertices): 1.83 ms
+// for the call against 1.70 on 4; 16 for rgg3d 77,488, k = 5 (930 vertices): 2.69 against
+// 2.53 on 8; and what this rule chooses, too, for 1,000,003, k = 64 (4: 9.7 ms, 6: 9.9, 8:
+// 12.2) and 4M, k = 64 (6: 23.0, 8: 26.1).
+constexpr long long kTiny = 512, kSmall = 4096;
+constexpr double kRelSmall[fr_ctx::kNumClusterSizes] = {1.17, 1.05, 1.0, 1.0, 1.0};
 // host staging offsets (the first megabytes of h_stage belong to the other paths)
 constexpr size_t kStageGraphs = 4u << 20;
 constexpr size_t kStagePrev = (4u << 20) + (64u << 10);
@@ -222,9 +235,10 @@ int queue_size_for(fr_ctx *ctx, const BatchPlan &pl, const fr_options *opt) {
             continue;
         }
         if (need > per_cta * c) continue;
-        // pairs in flight at once over the time of one pair
-        const double v = (double)std::min(ctx->q_cap[t], pl.np) / kRelTime[t];
-        if (best < 0 || v > bestv) { best = t; bestv = v; }
+        const double chain = pl.nr, turns = (double)pl.np / std::min(ctx->q_cap[t], pl.np);
+        const double v = est <= kTiny ? (double)c : std::sqrt(chain * chain + turns * turns) *
+                                                        (est <= kSmall ? kRelSmall : kRelTime)[t];
+        if (best < 0 || v < bestv) { best = t; bestv = v; }
     }
     return best;
 }
@@ -433,7 +447,6 @@ int queue_round_size(fr_ctx *ctx, int P, long long est, double avg_degree, const
     const double need = 1.05 * (double)est * (29.0 + 16.0 * avg_degree);
     const double per_cta = 0.95 * (double)queue_smem();
     const int force = opt->cluster_ctas ? opt->cluster_ctas : ctx->tune_ctas;
-    constexpr long long kTiny = 512;
     int best = -1, kept = -1;
     double bestc = 0, keptc = 0;
     for (int t = 0; t < fr_ctx::kNumClusterSizes; ++t) {
