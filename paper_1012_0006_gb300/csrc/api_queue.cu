@@ -221,8 +221,12 @@ int queue_size_for(fr_ctx *ctx, const BatchPlan &pl, const fr_options *opt) {
     if (dyn == 0) return -1;
     long long est = 0;
     for (long long e : pl.est_max) est = std::max(est, e);
+    // The workspace depends on the size, and with it which calls an arena bound admits: under a
+    // bound the size is the one with the most pairs in flight over a pair's time, whatever is
+    // fastest, so that no call is refused for speed.
+    const bool bounded = ctx->arena_limit != 0;
     // (16 bytes an arc: the arcs a slot has room for, see caps_for)
-    const double need = 1.05 * (double)est * (29.0 + 16.0 * pl.avg_degree);
+    const double need = 1.05 * (double)est * (29.0 + (bounded && !ctx->narrow_ok ? 20.0 : 16.0) * pl.avg_degree);
     const double per_cta = 0.95 * (double)dyn;
     const int force = opt->cluster_ctas ? opt->cluster_ctas : ctx->tune_ctas;
     int best = -1;
@@ -236,7 +240,8 @@ int queue_size_for(fr_ctx *ctx, const BatchPlan &pl, const fr_options *opt) {
         }
         if (need > per_cta * c) continue;
         const double chain = pl.nr, turns = (double)pl.np / std::min(ctx->q_cap[t], pl.np);
-        const double v = est <= kTiny ? (double)c : std::sqrt(chain * chain + turns * turns) *
+        const double v = bounded ? -(double)std::min(ctx->q_cap[t], pl.np) / kRelTime[t] :
+                         est <= kTiny ? (double)c : std::sqrt(chain * chain + turns * turns) *
                                                         (est <= kSmall ? kRelSmall : kRelTime)[t];
         if (best < 0 || v < bestv) { best = t; bestv = v; }
     }

@@ -126,7 +126,7 @@ def test_rounds_on_the_queue_kernel(F, ctx, dev, fm):
     _active(F, ctx, w, dev, **okw)
 
 
-@pytest.mark.parametrize("call", ["pair", "active"])
+@pytest.mark.parametrize("call", ["pair", "active", "batch"])
 def test_arena_bounds_between_the_workspaces(F, call):
     w = dict(I.grid2d_halves(128, 128, swaps=500, alpha=4.0), mb=1)
     w["part"] = I.rcb(I.grid2d(128, 128)[2], w["vwgt"], 4)
@@ -135,6 +135,8 @@ def test_arena_bounds_between_the_workspaces(F, call):
     okw = dict(mb=1)
     if call == "pair":
         st, pref, _ = O.refine_pair(w, 0, 1, opts=O.options(**okw))
+    elif call == "batch":
+        st, pref, _, _ = O.refine_batch(w, opts=O.options(**okw))
     else:
         st, pref, _, _ = O.refine_active(w, opts=O.options(**okw), max_outer=2)
     ran = []
@@ -143,6 +145,8 @@ def test_arena_bounds_between_the_workspaces(F, call):
         with F.Context(0, arena_bytes=mib << 20) as c:
             if call == "pair":
                 st, _ = c.refine_pair(g, part, 4, 0, 1, w["eps"], w["alpha"], F.default_options(**okw), check=False)
+            elif call == "batch":
+                st, *_ = c.refine_batch(g, part, 4, w["eps"], w["alpha"], F.default_options(**okw), check=False)
             else:
                 st, *_ = c.refine_active(g, part, 4, w["eps"], w["alpha"], F.default_options(**okw), max_outer=2,
                                          check=False)
