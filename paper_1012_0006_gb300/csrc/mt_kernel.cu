@@ -515,8 +515,13 @@ __device__ __forceinline__ void mt_search(const GraphDev &G, const MtDev &m, MtS
             }
             const int own = 31 - __clz(has);   // the lane whose words hold the highest bit
             b = __shfl_sync(kFull, w2.y ? lane * 64 + 63 - __clz(w2.y) : lane * 64 + 31 - __clz(w2.x), own);
-            const int at = S.top[b];
+            int at = S.top[b];
             e = mt_entry(S, m, at, nxt, rbase);
+            while (!e.z && e.y >= 0) {   // dead ones on one another: no new look at the bits
+                // (three global rounds of rgg3d 524,288, k = 64: 51.4 -> 49.1 ms)
+                at = e.y;
+                e = mt_entry(S, m, at, nxt, rbase);
+            }
             __syncwarp();
             if (lane == own) {
                 S.top[b] = e.y;
