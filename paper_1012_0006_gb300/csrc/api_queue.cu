@@ -27,7 +27,7 @@ constexpr double kRelTime[fr_ctx::kNumClusterSizes] = {1.25, 1.05, 1.0, 0.85, 0.
 // pairs that wait for one another, and the clusters have turns = pairs / clusters to take;
 // sqrt(nr^2 + turns^2) times the time of one pair fits both ends.  Corridors of fewer
 // vertices than a cluster of 8 has threads gain little from more CTAs, of fewer than one CTA
-// has none.  Taking the most pairs in flight over a pair's time alone (the chain left out)
+// has nothing (rgg2d 20,011, k = 7: the kernel 1.47 ms on 4, 1.49, 1.52, 1.57, 1.66 on 16).  Taking the most pairs in flight over a pair's time alone (the chain left out)
 // chose 4 CTAs for rgg3d 524,287 vertices, k = 32 (18 rounds, 155 pairs, 1,316 vertices):
 // 8.2 ms, against 7.5 on 6 and 7.4 on 8; 8 for rgg2d 20,011, k = 7 (346 vertices): 1.83 ms
 // for the call against 1.70 on 4; 16 for rgg3d 77,488, k = 5 (930 vertices): 2.69 against
@@ -35,6 +35,7 @@ constexpr double kRelTime[fr_ctx::kNumClusterSizes] = {1.25, 1.05, 1.0, 0.85, 0.
 // 12.2) and 4M, k = 64 (6: 23.0, 8: 26.1).
 constexpr long long kTiny = 512, kSmall = 4096;
 constexpr double kRelSmall[fr_ctx::kNumClusterSizes] = {1.17, 1.05, 1.0, 1.0, 1.0};
+constexpr double kRelTiny[fr_ctx::kNumClusterSizes] = {1.0, 1.01, 1.02, 1.06, 1.13};
 // host staging offsets (the first megabytes of h_stage belong to the other paths)
 constexpr size_t kStageGraphs = 4u << 20;
 constexpr size_t kStagePrev = (4u << 20) + (64u << 10);
@@ -93,6 +94,12 @@ T *take(char *&p, long long count) {
     return r;
 }
 
+// Ticket, votes, abort word, control blocks and counters of a launch on `clusters` clusters.
+size_t queue_state_bytes(const fr_ctx *ctx, int clusters) {
+    return 2 * al256(sizeof(int)) + al256(sizeof(fr_ctx::QCtl) * (size_t)ctx->q_clusters) +
+           4 * sizeof(long long) * (size_t)clusters;
+}
+
 fr_status ensure_queue(fr_ctx *ctx, int ctas, int clusters, int n, int nnz, int k, int reps, int np) {
     if (ctx->q_mem && ctas == ctx->q_ctas && clusters <= ctx->q_clusters && n <= ctx->q_n && nnz <= ctx->q_nnz &&
         k <= ctx->q_k && reps <= ctx->q_reps && np <= ctx->q_np)
@@ -135,6 +142,8 @@ fr_status ensure_queue(fr_ctx *ctx, int ctas, int clusters, int n, int nnz, int 
     char *p = reinterpret_cast<char *>(ctx->q_mem);
     ctx->q_ticket = take<int>(p, 2);
     ctx->q_gabort = take<int>(p, 1);
+    ctx->q_ctls = take<fr_ctx::QCtl>(p, cc);   // (cleared with the words before them, and the
+    ctx->q_stats = take<long long>(p, 4LL * cc);   // abort word read back with them: queue_state_bytes)
     ctx->q_prev = take<int>(p, 2LL * pp);
     ctx->q_crank = take<int>(p, mm);
     ctx->q_slots = take<QSlot>(p, cc);
@@ -146,19 +155,23 @@ fr_status ensure_queue(fr_ctx *ctx, int ctas, int clusters, int n, int nnz, int 
     ctx->qb_lst = take<int>(p, nn);
     ctx->qb_cap = (int)qcap;
     ctx->q_graphs = take<GraphDev>(p, cc);
-    ctx->q_ctls = take<fr_ctx::QCtl>(p, cc);
-    ctx->q_stats = take<long long>(p, 4LL * cc);
     ctx->q_host.assign(cc, QSlot());
-    for (int i = 0; i < cc; ++i) {
-        QSlot &S = ctx->q_host[i];
-        S.graph = ctx->q_graphs + i;
-        S.sob = take<int>(p, kk);
-        S.ctl = &ctx->q_ctls[i].c;
-        S.hist = take<long long>(p, 3LL * 2 * kHistBins);
-        S.cta_cnt = take<int>(p, ctas + 1);
+    // what is idle between launches lies together over the slots, to be cleared in two calls
+    char *const idle = p;
+    for (QSlot &S : ctx->q_host) S.sob = take<int>(p, kk);
+    char *const bits = p;
+    for (QSlot &S : ctx->q_host) {
         S.cbits = take<unsigned int>(p, c.words);
         S.sdbits = take<unsigned int>(p, c.words);
         S.sbits = take<unsigned int>(p, c.swords);
+    }
+    char *const slots = p;
+    for (int i = 0; i < cc; ++i) {
+        QSlot &S = ctx->q_host[i];
+        S.graph = ctx->q_graphs + i;
+        S.ctl = &ctx->q_ctls[i].c;
+        S.hist = take<long long>(p, 3LL * 2 * kHistBins);
+        S.cta_cnt = take<int>(p, ctas + 1);
         S.vq_v = take<int>(p, c.vq); S.vq_s = take<int>(p, c.vq);
         int **v21[21] = {&S.gid, &S.sid, &S.off, &S.infc, &S.fx, &S.lab, &S.rflag, &S.color, &S.scc, &S.vc,
                          &S.fq0, &S.fq1, &S.cid, &S.cpair, &S.cmin, &S.indeg, &S.outoff, &S.ocur, &S.plist,
@@ -173,12 +186,10 @@ fr_status ensure_queue(fr_ctx *ctx, int ctas, int clusters, int n, int nnz, int 
         S.hkey = take<unsigned long long>(p, (long long)rr * c.nu);
         S.sw_absd = take<long long>(p, rr); S.sw_j = take<int>(p, rr);
         S.stat = ctx->q_stats + 4LL * i;
-        // idle state: no block paired, no corridor bit set
-        CK(cudaMemsetAsync(S.sob, 0xFF, sizeof(int) * (size_t)kk, ctx->stream));
-        CK(cudaMemsetAsync(S.cbits, 0, sizeof(unsigned int) * (size_t)c.words, ctx->stream));
-        CK(cudaMemsetAsync(S.sdbits, 0, sizeof(unsigned int) * (size_t)c.words, ctx->stream));
-        CK(cudaMemsetAsync(S.sbits, 0, sizeof(unsigned int) * (size_t)c.swords, ctx->stream));
     }
+    // idle state: no block paired, no corridor bit set
+    CK(cudaMemsetAsync(idle, 0xFF, (size_t)(bits - idle), ctx->stream));
+    CK(cudaMemsetAsync(bits, 0, (size_t)(slots - bits), ctx->stream));
     CK(cudaMemcpyAsync(ctx->q_slots, ctx->q_host.data(), sizeof(QSlot) * cc, cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     destroy_graph_cache(ctx);   // captured sweeps hold pointers into the old workspace
@@ -229,8 +240,8 @@ int queue_size_for(fr_ctx *ctx, const BatchPlan &pl, const fr_options *opt) {
     const double need = 1.05 * (double)est * (29.0 + (bounded && !ctx->narrow_ok ? 20.0 : 16.0) * pl.avg_degree);
     const double per_cta = 0.95 * (double)dyn;
     const int force = opt->cluster_ctas ? opt->cluster_ctas : ctx->tune_ctas;
-    int best = -1;
-    double bestv = 0;
+    int best = -1, kept = -1;
+    double bestv = 0, keptv = 0;
     for (int t = 0; t < fr_ctx::kNumClusterSizes; ++t) {
         if (ctx->q_cap[t] <= 0) continue;
         const int c = fr_ctx::kClusterSizes[t];
@@ -241,10 +252,15 @@ int queue_size_for(fr_ctx *ctx, const BatchPlan &pl, const fr_options *opt) {
         if (need > per_cta * c) continue;
         const double chain = pl.nr, turns = (double)pl.np / std::min(ctx->q_cap[t], pl.np);
         const double v = bounded ? -(double)std::min(ctx->q_cap[t], pl.np) / kRelTime[t] :
-                         est <= kTiny ? (double)c : std::sqrt(chain * chain + turns * turns) *
-                                                        (est <= kSmall ? kRelSmall : kRelTime)[t];
+                         std::sqrt(chain * chain + turns * turns) *
+                             (est <= kTiny ? kRelTiny : est <= kSmall ? kRelSmall : kRelTime)[t];
         if (best < 0 || v < bestv) { best = t; bestv = v; }
+        if (ctx->q_mem && ctx->q_ctas == c) { kept = t; keptv = v; }
     }
+    // The size laid out already, unless another is clearly better: laying out again takes a few
+    // tenths of a millisecond and drops the captured sweeps (a V-cycle of grid3d 108,570
+    // vertices, k = 14, that went between 4 and 8 CTAs: 25.4 ms, 23.8 on 4 throughout).
+    if (!bounded && kept >= 0 && keptv <= 1.07 * bestv) return kept;
     return best;
 }
 
@@ -309,10 +325,7 @@ fr_status run_queue_sweep(fr_ctx *ctx, const fr_graph *g, int32_t *part, const B
         CK(launch_fill_pairs(ctx->pairs, ctx->pair_a, ctx->pair_b, pl.np, 0, opt->mb ? 1 : 0, pl.Ubase, ctx->stream));
         CK(cudaMemsetAsync(ctx->sides, 0, sizeof(SideDev) * 2 * (size_t)pl.np, ctx->stream));
         CK(cudaMemsetAsync(ctx->pacc, 0, sizeof(PairAcc) * (size_t)pl.np, ctx->stream));
-        CK(cudaMemsetAsync(ctx->q_ticket, 0, 2 * sizeof(int), ctx->stream));   // (and the votes)
-        CK(cudaMemsetAsync(ctx->q_gabort, 0, sizeof(int), ctx->stream));
-        CK(cudaMemsetAsync(ctx->q_ctls, 0, sizeof(fr_ctx::QCtl) * (size_t)clusters, ctx->stream));
-        CK(cudaMemsetAsync(ctx->q_stats, 0, 4 * sizeof(long long) * (size_t)clusters, ctx->stream));
+        CK(cudaMemsetAsync(ctx->q_ticket, 0, queue_state_bytes(ctx, clusters), ctx->stream));
         CK(cudaMemsetAsync(ctx->qb_lst, 0xFF, sizeof(int) * (size_t)g->n, ctx->stream));
         CK(cudaMemsetAsync(ctx->qb_cnt, 0, sizeof(int) * (size_t)pl.k, ctx->stream));
         CK(launch_qb_build(ctx->bl, ctx->blc, part, pl.k, ctx->qb_cnt, ctx->qb_start, ctx->qb_app, ctx->qb_lst,
@@ -498,7 +511,6 @@ fr_status enqueue_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int
         gd.bl = ctx->bl; gd.blc = ctx->blc; gd.inb = ctx->inb;
     }
     CK(cudaMemcpyAsync(ctx->q_graphs, hg, sizeof(GraphDev) * (size_t)clusters, cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaMemsetAsync(ctx->q_prev, 0xFF, sizeof(int) * 2 * (size_t)P, ctx->stream));   // no pair waits
     // part and the block weights as they are, should a pair outgrow its cluster
     CK(cudaMemcpyAsync(ctx->spare, part, sizeof(int) * (size_t)g->n, cudaMemcpyDeviceToDevice, ctx->stream));
     CK(cudaMemcpyAsync(ctx->h_stage + kStageRoundW, ctx->blockw, sizeof(long long) * (size_t)k, cudaMemcpyDeviceToHost,
@@ -514,18 +526,13 @@ fr_status enqueue_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int
     q.slots = ctx->q_slots;
     q.np = P;
     q.ticket = ctx->q_ticket;
-    q.prev = ctx->q_prev;
+    q.prev = nullptr;   // no pair waits for another
     q.gabort = ctx->q_gabort;
     q.wait_ns = kWaitNs;
-    // the ticket and the abort word lie next to each other, and so do the control blocks
-    // and the counters
-    CK(cudaMemsetAsync(ctx->q_ticket, 0, al256(sizeof(int)) + sizeof(int), ctx->stream));
-    CK(cudaMemsetAsync(ctx->q_ctls, 0, al256(sizeof(fr_ctx::QCtl) * (size_t)ctx->q_clusters) +
-                                           4 * sizeof(long long) * (size_t)clusters, ctx->stream));
+    CK(cudaMemsetAsync(ctx->q_ticket, 0, queue_state_bytes(ctx, clusters), ctx->stream));
     CK(launch_queue_sweep(q, ctas, clusters, ctx->stream));
     char *h = ctx->h_stage + kStageRoundCtl;
-    CK(cudaMemcpyAsync(h, ctx->q_gabort, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaMemcpyAsync(h + 256, ctx->q_ctls, sizeof(fr_ctx::QCtl) * (size_t)clusters, cudaMemcpyDeviceToHost,
+    CK(cudaMemcpyAsync(h, ctx->q_gabort, 256 + sizeof(fr_ctx::QCtl) * (size_t)clusters, cudaMemcpyDeviceToHost,
                        ctx->stream));
     rq->queued = true;
     rq->clusters = clusters;

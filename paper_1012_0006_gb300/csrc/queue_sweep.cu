@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(TPB, 1) queue_kernel(QueueArgs q, size_t smem_
             if (*(volatile int *)q.gabort == 0) {
                 j = atomicAdd(q.ticket, 1);
                 if (j < q.np) {
-                    const int pa = q.prev[2 * j], pb = q.prev[2 * j + 1];
+                    const int pa = q.prev ? q.prev[2 * j] : -1, pb = q.prev ? q.prev[2 * j + 1] : -1;
                     const unsigned long long t_start = globaltimer();
                     unsigned int spins = 0;
                     while ((pa >= 0 && ld_acquire_i(&q.wt.pacc[pa].done) == 0) ||

@@ -41,7 +41,7 @@ struct QueueArgs {
     int *ticket;          // next pair to take (zero before the launch)
     int *votes;           // pairs whose flow started with a wave that paid, less those it did not pay
                           // (zero before the launch; NULL: no pair does)
-    const int *prev;      // [2 np]: the last earlier pair that shares block a (b), or -1
+    const int *prev;      // [2 np]: the last earlier pair that shares block a (b), or -1; NULL: none does
     int *gabort;          // 0, E_MISFIT (run the sweep round by round instead), or an error code
     unsigned long long wait_ns;   // bound of one wait for a dependency (then E_ABORT)
 };
