@@ -6,13 +6,13 @@
 // The round's persistent kernel builds every pair's corridor network in HBM.  This
 // kernel then gives each pair one cluster of C CTAs: the pair's vertices are split
 // into C contiguous ranges with about equal arc counts, and every CTA loads its
-// range -- labels, excess, s/t-arc flow, CSR offsets, the shared::cluster addresses
-// of each arc's head label and reverse residual, residual capacities -- into its
-// shared memory.  Push-relabel (lock-free pulses, or waves by levels), the exact
-// relabels, the reachability sets and the SCCs then run on shared memory with the
-// cluster's hardware barrier (~0.3 us) instead of a grid barrier (~3 us).  No CTA
-// reads another's vertex state in these loops: updates travel as remote stores and
-// relaxed reductions into the owner's memory, and each arc keeps a copy of its head's
+// range -- labels, excess, s/t-arc flow, CSR offsets, and 8 bytes per arc with the
+// places of its head and its reverse arc and its residual -- into its shared memory.
+// Push-relabel (pulses, or waves by levels), the exact relabels, the reachability sets
+// and the SCCs then run on shared memory with the cluster's hardware barrier (~0.25 us)
+// instead of a grid barrier (~3 us).  No CTA reads another's vertex state in these
+// loops: updates for another CTA are queued and sent together as relaxed reductions and
+// stores into the owner's memory, and an arc to another CTA has a copy of its head's
 // label that the head publishes.  Results go back to HBM for the DAG and sweep
 // phases.  A pair whose network does not fit is left to a second launch with larger
 // clusters, then to the grid-wide path (ctl->fallback).
