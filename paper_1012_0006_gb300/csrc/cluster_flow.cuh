@@ -20,6 +20,11 @@ namespace cg = cooperative_groups;
 
 constexpr int kClusterMax = 16;
 constexpr int kHdrBytes = 1024;
+// A network of up to this many vertices stays in one CTA of its cluster: fewer vertices than
+// the CTA has threads are not worth the updates that cross CTAs.  Split, 128 and 384: the pair
+// of the 64 x 64 grid 308, 293, 285 us; a V-cycle of rgg3d 1,000,003 vertices, k = 64, 69.1,
+// 67.4, 67.0 ms; a W-cycle of rgg3d 65,536, k = 64, 97.3, 93.6, 93.5 ms.
+constexpr int kWhole = 384;
 
 struct ClusterHdr {
     int klo[kClusterMax + 1];   // member ranges of the CTAs (identical in every CTA)
@@ -490,9 +495,10 @@ struct ClusterFlow {
                 pick = c;
                 if (bytes_for(nvc, nac, w.narrow != 0) <= smem_bytes) break;
             }
+            const bool whole = V <= kWhole && bytes_for(V, A, w.narrow != 0) <= smem_bytes;
             for (int r = 0; r <= C; ++r) {
-                H()->klo[r] = H()->kloc[pick][r];
-                H()->cab[r] = H()->cabc[pick][r];
+                H()->klo[r] = whole && r > 0 ? V : H()->kloc[pick][r];
+                H()->cab[r] = whole && r > 0 ? A : H()->cabc[pick][r];
             }
         }
         sync();

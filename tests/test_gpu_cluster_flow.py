@@ -95,7 +95,7 @@ def test_rows_of_every_length(F, ctx, deg_lo, deg_hi, ctas):
 
 
 @pytest.mark.parametrize("scale", [1, 3000, 5000])
-@pytest.mark.parametrize("n,deg", [(600, 4), (2000, 12), (5000, 20)])
+@pytest.mark.parametrize("n,deg", [(600, 4), (957, 4), (960, 6), (963, 8), (2000, 12), (5000, 20)])
 def test_networks_that_cross_ctas(F, ctx, n, deg, scale):
     w = _random_regular(n, deg, scale)
     for dev in (dict(cluster_ctas=4), dict(cluster_ctas=16), dict(sweep_sched=1)):
