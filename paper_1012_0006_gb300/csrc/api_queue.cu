@@ -94,7 +94,7 @@ T *take(char *&p, long long count) {
     return r;
 }
 
-// Ticket, votes, abort word, control blocks and counters of a launch on `clusters` clusters.
+// Ticket, votes, scan length, abort word, control blocks and counters of a launch on `clusters` clusters.
 size_t queue_state_bytes(const fr_ctx *ctx, int clusters) {
     return 2 * al256(sizeof(int)) + al256(sizeof(fr_ctx::QCtl) * (size_t)ctx->q_clusters) +
            4 * sizeof(long long) * (size_t)clusters;
@@ -140,7 +140,7 @@ fr_status ensure_queue(fr_ctx *ctx, int ctas, int clusters, int n, int nnz, int 
     ctx->q_np = pp;
     ctx->q_nu = c.nu; ctx->q_mu = c.mu; ctx->q_vq = c.vq;
     char *p = reinterpret_cast<char *>(ctx->q_mem);
-    ctx->q_ticket = take<int>(p, 2);
+    ctx->q_ticket = take<int>(p, 3);   // ticket, votes, scan length
     ctx->q_gabort = take<int>(p, 1);
     ctx->q_ctls = take<fr_ctx::QCtl>(p, cc);   // (cleared with the words before them, and the
     ctx->q_stats = take<long long>(p, 4LL * cc);   // abort word read back with them: queue_state_bytes)
@@ -530,6 +530,10 @@ fr_status enqueue_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int
     q.gabort = ctx->q_gabort;
     q.wait_ns = kWaitNs;
     CK(cudaMemsetAsync(ctx->q_ticket, 0, queue_state_bytes(ctx, clusters), ctx->stream));
+    if (P > 1) {   // pairs commit to the list while others scan it: they scan what is on it now
+        q.wt.scan_len = ctx->q_ticket + 2;
+        CK(cudaMemcpyAsync(ctx->q_ticket + 2, ctx->blc, sizeof(int), cudaMemcpyDeviceToDevice, ctx->stream));
+    }
     CK(launch_queue_sweep(q, ctas, clusters, ctx->stream));
     char *h = ctx->h_stage + kStageRoundCtl;
     CK(cudaMemcpyAsync(h, ctx->q_gabort, 256 + sizeof(fr_ctx::QCtl) * (size_t)clusters, cudaMemcpyDeviceToHost,

@@ -275,7 +275,10 @@ struct StepKernel {
             }
             cnt = seg[0] + seg[1] + seg[2] + seg[3];
         } else {
-            cnt = __ldcg(Gr.blc);
+            // (beside the scan, another cluster's commit may append: first the count grows, then
+            // the entry is written.  Such an entry is a vertex of that pair's blocks, no
+            // candidate of this pair, so the length at the round's start is all it needs.)
+            cnt = __ldcg(w.scan_len ? w.scan_len : Gr.blc);
         }
         long long n_rows = 0, n_arcs = 0, cut = 0;
         for (long long base = G.warp * 32; base < cnt; base += G.nwarps * 32) {
