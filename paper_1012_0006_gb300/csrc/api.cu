@@ -498,7 +498,8 @@ extern "C" fr_status fr_destroy(fr_ctx *ctx) {
     free_pairs(ctx);
     free_fm(ctx);
     free_mt(ctx);
-    free_queue(ctx);
+    free_queue(ctx->sweep_q);
+    free_queue(ctx->round_q);
     if (ctx->reps_mem) cudaFree(ctx->reps_mem);
     if (ctx->hg_mem) cudaFree(ctx->hg_mem);
     if (ctx->h_stage) cudaFreeHost(ctx->h_stage);

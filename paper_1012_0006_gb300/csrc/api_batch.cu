@@ -593,7 +593,7 @@ static fr_status batch_core(fr_ctx *ctx, const fr_graph *g, int32_t *part, int32
     CK(cudaMemcpyAsync(S.data(), ctx->sides, sizeof(SideDev) * 2 * pl.np, cudaMemcpyDeviceToHost, ctx->stream));
     std::vector<long long> qst(queued ? 4 * ctx->last_queue_clusters : 0);
     if (!qst.empty())
-        CK(cudaMemcpyAsync(qst.data(), ctx->q_stats, sizeof(long long) * qst.size(), cudaMemcpyDeviceToHost,
+        CK(cudaMemcpyAsync(qst.data(), ctx->sweep_q.stats, sizeof(long long) * qst.size(), cudaMemcpyDeviceToHost,
                            ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     fr_status bad = FR_OK;

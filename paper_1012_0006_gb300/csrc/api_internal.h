@@ -21,6 +21,29 @@ struct GraphCacheEntry {
     long long launches = 0;   // kernels in the captured sweep
 };
 
+// Workspace of one launch of the queue kernel: the slots of its clusters, laid out for the
+// last cluster size used and the largest sizes seen with it (allocated on first use).
+struct QueueMem {
+    void *mem = nullptr;
+    size_t bytes = 0;
+    int ctas = 0, clusters = 0, n = 0, nnz = 0, k = 0, reps = 0, np = 0;
+    long long nu = 0, mu = 0, vq = 0;
+    fr::QSlot *slots = nullptr;                // device array [clusters]
+    std::vector<fr::QSlot> host;               // the same descriptors on the host
+    // the slots' graph descriptors, control blocks and counters, each array contiguous so
+    // that a launch sets and reads them with one copy apiece
+    fr::GraphDev *graphs = nullptr;
+    struct alignas(256) QCtl { fr::Ctl c; };   // one control block per 256 bytes: no line shared by two clusters
+    QCtl *ctls = nullptr;
+    long long *stats = nullptr;                // [4 clusters]
+    int *ticket = nullptr, *gabort = nullptr, *crank = nullptr;
+    // sweeps only: the pairs' predecessors, the candidate lists per block
+    int *prev = nullptr;
+    int *qb_sorted = nullptr, *qb_start = nullptr, *qb_cnt = nullptr, *qb_app = nullptr, *qb_pool = nullptr,
+        *qb_lst = nullptr;
+    int qb_cap = 0;
+};
+
 struct fr_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -113,26 +136,10 @@ struct fr_ctx {
     fr_profile_info prof = {};
     std::vector<float> round_ms;   // per round: scan, step 1, cluster kernels, step 2 (profiling)
     std::vector<float> pair_ms;    // per pair: round, cluster start and end after the round's first start
-    // queue sweep (every pair of a sweep in one launch of clusters, see queue_sweep.cu):
-    // resident clusters of the queue kernel per cluster size, and the per-cluster
-    // workspaces of the last size used (allocated on first use)
+    // queue kernel (queue_sweep.cu): resident clusters per cluster size, and the workspaces of
+    // its launches: one for sweeps, one for single rounds (pairs, active scheduling)
     int q_cap[kNumClusterSizes] = {0, 0, 0, 0, 0};
-    void *q_mem = nullptr;
-    size_t q_bytes = 0;
-    int q_ctas = 0, q_clusters = 0, q_n = 0, q_nnz = 0, q_k = 0, q_reps = 0, q_np = 0;
-    long long q_nu = 0, q_mu = 0, q_vq = 0;
-    fr::QSlot *q_slots = nullptr;              // device array [q_clusters]
-    std::vector<fr::QSlot> q_host;             // the same descriptors on the host
-    // the slots' graph descriptors, control blocks and counters, each array contiguous so
-    // that a sweep sets and reads them with one copy apiece
-    fr::GraphDev *q_graphs = nullptr;
-    struct alignas(256) QCtl { fr::Ctl c; };   // one control block per 256 bytes: no line shared by two clusters
-    QCtl *q_ctls = nullptr;
-    long long *q_stats = nullptr;              // [4 q_clusters]
-    int *q_ticket = nullptr, *q_gabort = nullptr, *q_prev = nullptr, *q_crank = nullptr;
-    int *qb_sorted = nullptr, *qb_start = nullptr, *qb_cnt = nullptr, *qb_app = nullptr, *qb_pool = nullptr,
-        *qb_lst = nullptr;
-    int qb_cap = 0;
+    QueueMem sweep_q, round_q;
     bool last_queue = false;                   // the last fr_refine_batch ran as a queue sweep
     int last_queue_ctas = 0, last_queue_clusters = 0, queue_fallbacks = 0;
 };
@@ -204,7 +211,7 @@ cudaError_t launch_round(fr_ctx *ctx, fr::Work &w, int grid, int tpb, cudaStream
 cudaError_t launch_clusters(fr_ctx *ctx, fr::Work &w, long long est_pair_vertices, double avg_degree, int force,
                             cudaStream_t st, int *nl);
 void release_corridor(fr_ctx *ctx);
-void free_queue(fr_ctx *ctx);
+void free_queue(QueueMem &Q);
 // Index into fr_ctx::kClusterSizes of the queue sweep's cluster size for plan pl, or -1
 // when the queue does not apply (FM step, no cluster capacity, estimate beyond 16 CTAs).
 int queue_size_for(fr_ctx *ctx, const BatchPlan &pl, const fr_options *opt);

@@ -94,82 +94,101 @@ T *take(char *&p, long long count) {
     return r;
 }
 
-// Ticket, votes, scan length, abort word, control blocks and counters of a launch on `clusters` clusters.
-size_t queue_state_bytes(const fr_ctx *ctx, int clusters) {
-    return 2 * al256(sizeof(int)) + al256(sizeof(fr_ctx::QCtl) * (size_t)ctx->q_clusters) +
+// Ticket, votes, scan length, abort word, control blocks and counters of a launch on
+// `clusters` clusters.
+size_t queue_state_bytes(const QueueMem &Q, int clusters) {
+    return 2 * al256(sizeof(int)) + al256(sizeof(QueueMem::QCtl) * (size_t)Q.clusters) +
            4 * sizeof(long long) * (size_t)clusters;
 }
 
-fr_status ensure_queue(fr_ctx *ctx, int ctas, int clusters, int n, int nnz, int k, int reps, int np) {
-    if (ctx->q_mem && ctas == ctx->q_ctas && clusters <= ctx->q_clusters && n <= ctx->q_n && nnz <= ctx->q_nnz &&
-        k <= ctx->q_k && reps <= ctx->q_reps && np <= ctx->q_np)
+// Entries of a block's region for the commits' appends (a sweep that fills one runs again
+// round by round).
+long long qb_cap_for(int n, int k) { return std::max<long long>(4096, 8LL * ((n + k - 1) / k)); }
+
+// lists: a sweep's predecessors and per-block candidate lists (24 to 40 bytes a vertex), which
+// a single round does not read.
+size_t queue_bytes(int ctas, int clusters, int n, int nnz, int k, int reps, int np, bool lists) {
+    size_t b = 2 * al256(4) + al256(4ull * nnz) + al256(sizeof(QSlot) * clusters) + al256(sizeof(GraphDev) * clusters) +
+               al256(sizeof(QueueMem::QCtl) * clusters) + al256(32ull * clusters) +
+               slot_bytes(caps_for(ctas, n), ctas, k, reps) * clusters;
+    if (lists)
+        b += al256(8ull * np) + 2 * al256(4ull * n) + al256(4ull * (k + 1)) + 2 * al256(4ull * k) +
+             al256(4ull * k * qb_cap_for(n, k));
+    return b;
+}
+
+// Lays Q out for launches on up to `clusters` clusters of `ctas` CTAs.  Sweeps and rounds have
+// a workspace each: a program that calls both would lay a shared one out again at every change
+// of cluster size, and drop its captured sweeps with it (a sweep of rgg2d 20,011, k = 7, in turn
+// with a pair of 65,536 vertices: 1.97 ms, 1.90 with two), and a sweep under an arena bound
+// could be refused for the sizes that a pair call before it had asked for.
+fr_status ensure_queue(fr_ctx *ctx, QueueMem &Q, int ctas, int clusters, int n, int nnz, int k, int reps, int np) {
+    if (Q.mem && ctas == Q.ctas && clusters <= Q.clusters && n <= Q.n && nnz <= Q.nnz && k <= Q.k && reps <= Q.reps &&
+        np <= Q.np)
         return FR_OK;
-    const int nn = std::max(n, ctx->q_ctas == ctas ? ctx->q_n : 0);
-    const int mm = std::max(nnz, ctx->q_ctas == ctas ? ctx->q_nnz : 0);
-    const int kk = std::max(k, ctx->q_ctas == ctas ? ctx->q_k : 0);
-    const int rr = std::max(reps, ctx->q_ctas == ctas ? ctx->q_reps : 1);
-    const int pp = std::max(np, ctx->q_ctas == ctas ? ctx->q_np : 0);
-    const int cc = std::max(clusters, ctx->q_ctas == ctas ? ctx->q_clusters : 0);
-    const QCaps c = caps_for(ctas, nn);
-    const size_t per = slot_bytes(c, ctas, kk, rr);
-    // per-block candidate lists: the sweep's candidates bucketed, and a region per block
-    // for the commits' appends (a sweep that fills one runs again round by round)
-    const long long qcap = std::max<long long>(4096, 8LL * ((nn + kk - 1) / kk));
-    size_t bytes = al256(4) + al256(4) + al256(8ull * pp) + al256(4ull * mm) + al256(sizeof(QSlot) * cc) +
-                   al256(sizeof(GraphDev) * cc) + al256(sizeof(fr_ctx::QCtl) * cc) + al256(32ull * cc) + per * cc +
-                   al256(4ull * nn) + al256(4ull * (kk + 1)) + 2 * al256(4ull * kk) + al256(4ull * kk * qcap) +
-                   al256(4ull * nn);
-    if (ctx->arena_limit && bytes + ctx->base_bytes + ctx->pair_bytes + ctx->reps_bytes > ctx->arena_limit) {
+    const bool sweep = &Q == &ctx->sweep_q;
+    const bool same = Q.ctas == ctas;
+    const int nn = std::max(n, same ? Q.n : 0), mm = std::max(nnz, same ? Q.nnz : 0), kk = std::max(k, same ? Q.k : 0);
+    const int rr = std::max(reps, same ? Q.reps : 1), pp = std::max(np, same ? Q.np : 0);
+    const int cc = std::max(clusters, same ? Q.clusters : 0);
+    const size_t bytes = queue_bytes(ctas, cc, nn, mm, kk, rr, pp, sweep);
+    // A round's workspace is taken where it fits beside the sweeps' (its launches have another
+    // form), and makes room for theirs.
+    const size_t others = ctx->base_bytes + ctx->pair_bytes + ctx->reps_bytes + (sweep ? 0 : ctx->sweep_q.bytes);
+    if (ctx->arena_limit && bytes + others > ctx->arena_limit) {
         ctx_error(ctx, "queue sweep workspace exceeds the arena bound");
         return FR_ERR_OOM;
     }
+    if (sweep && ctx->arena_limit && bytes + others + ctx->round_q.bytes > ctx->arena_limit) free_queue(ctx->round_q);
     // Another cluster size lays the same memory out again where it is large enough: a V-cycle
     // and the rounds of active scheduling change sizes often, and a cudaFree and cudaMalloc
     // pair takes longer than a small round.
-    if (!ctx->q_mem || bytes > ctx->q_bytes) {
-        free_queue(ctx);
-        if (cudaMalloc(&ctx->q_mem, bytes) != cudaSuccess) {
+    if (!Q.mem || bytes > Q.bytes) {
+        free_queue(Q);
+        if (cudaMalloc(&Q.mem, bytes) != cudaSuccess) {
             cudaGetLastError();
-            ctx->q_mem = nullptr;
+            Q.mem = nullptr;
             ctx_error(ctx, "cudaMalloc(%zu) for the queue sweep failed", bytes);
             return FR_ERR_OOM;
         }
-        ctx->q_bytes = bytes;
+        Q.bytes = bytes;
     }
-    ctx->q_ctas = ctas; ctx->q_clusters = cc; ctx->q_n = nn; ctx->q_nnz = mm; ctx->q_k = kk; ctx->q_reps = rr;
-    ctx->q_np = pp;
-    ctx->q_nu = c.nu; ctx->q_mu = c.mu; ctx->q_vq = c.vq;
-    char *p = reinterpret_cast<char *>(ctx->q_mem);
-    ctx->q_ticket = take<int>(p, 3);   // ticket, votes, scan length
-    ctx->q_gabort = take<int>(p, 1);
-    ctx->q_ctls = take<fr_ctx::QCtl>(p, cc);   // (cleared with the words before them, and the
-    ctx->q_stats = take<long long>(p, 4LL * cc);   // abort word read back with them: queue_state_bytes)
-    ctx->q_prev = take<int>(p, 2LL * pp);
-    ctx->q_crank = take<int>(p, mm);
-    ctx->q_slots = take<QSlot>(p, cc);
-    ctx->qb_sorted = take<int>(p, nn);
-    ctx->qb_start = take<int>(p, kk + 1);
-    ctx->qb_cnt = take<int>(p, kk);
-    ctx->qb_app = take<int>(p, kk);
-    ctx->qb_pool = take<int>(p, (long long)kk * qcap);
-    ctx->qb_lst = take<int>(p, nn);
-    ctx->qb_cap = (int)qcap;
-    ctx->q_graphs = take<GraphDev>(p, cc);
-    ctx->q_host.assign(cc, QSlot());
+    const QCaps c = caps_for(ctas, nn);
+    Q.ctas = ctas; Q.clusters = cc; Q.n = nn; Q.nnz = mm; Q.k = kk; Q.reps = rr; Q.np = pp;
+    Q.nu = c.nu; Q.mu = c.mu; Q.vq = c.vq;
+    char *p = reinterpret_cast<char *>(Q.mem);
+    Q.ticket = take<int>(p, 3);   // ticket, votes, scan length
+    Q.gabort = take<int>(p, 1);
+    Q.ctls = take<QueueMem::QCtl>(p, cc);   // (cleared with the words before them, and the
+    Q.stats = take<long long>(p, 4LL * cc);   // abort word read back with them: queue_state_bytes)
+    Q.crank = take<int>(p, mm);
+    Q.slots = take<QSlot>(p, cc);
+    if (sweep) {
+        Q.prev = take<int>(p, 2LL * pp);
+        Q.qb_sorted = take<int>(p, nn);
+        Q.qb_start = take<int>(p, kk + 1);
+        Q.qb_cnt = take<int>(p, kk);
+        Q.qb_app = take<int>(p, kk);
+        Q.qb_cap = (int)qb_cap_for(nn, kk);
+        Q.qb_pool = take<int>(p, (long long)kk * Q.qb_cap);
+        Q.qb_lst = take<int>(p, nn);
+    }
+    Q.graphs = take<GraphDev>(p, cc);
+    Q.host.assign(cc, QSlot());
     // what is idle between launches lies together over the slots, to be cleared in two calls
     char *const idle = p;
-    for (QSlot &S : ctx->q_host) S.sob = take<int>(p, kk);
+    for (QSlot &S : Q.host) S.sob = take<int>(p, kk);
     char *const bits = p;
-    for (QSlot &S : ctx->q_host) {
+    for (QSlot &S : Q.host) {
         S.cbits = take<unsigned int>(p, c.words);
         S.sdbits = take<unsigned int>(p, c.words);
         S.sbits = take<unsigned int>(p, c.swords);
     }
     char *const slots = p;
     for (int i = 0; i < cc; ++i) {
-        QSlot &S = ctx->q_host[i];
-        S.graph = ctx->q_graphs + i;
-        S.ctl = &ctx->q_ctls[i].c;
+        QSlot &S = Q.host[i];
+        S.graph = Q.graphs + i;
+        S.ctl = &Q.ctls[i].c;
         S.hist = take<long long>(p, 3LL * 2 * kHistBins);
         S.cta_cnt = take<int>(p, ctas + 1);
         S.vq_v = take<int>(p, c.vq); S.vq_s = take<int>(p, c.vq);
@@ -185,24 +204,24 @@ fr_status ensure_queue(fr_ctx *ctx, int ctas, int clusters, int n, int nnz, int 
         S.hcomp = take<int>(p, (long long)rr * c.nu);
         S.hkey = take<unsigned long long>(p, (long long)rr * c.nu);
         S.sw_absd = take<long long>(p, rr); S.sw_j = take<int>(p, rr);
-        S.stat = ctx->q_stats + 4LL * i;
+        S.stat = Q.stats + 4LL * i;
     }
     // idle state: no block paired, no corridor bit set
     CK(cudaMemsetAsync(idle, 0xFF, (size_t)(bits - idle), ctx->stream));
     CK(cudaMemsetAsync(bits, 0, (size_t)(slots - bits), ctx->stream));
-    CK(cudaMemcpyAsync(ctx->q_slots, ctx->q_host.data(), sizeof(QSlot) * cc, cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaMemcpyAsync(Q.slots, Q.host.data(), sizeof(QSlot) * cc, cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    destroy_graph_cache(ctx);   // captured sweeps hold pointers into the old workspace
+    if (sweep) destroy_graph_cache(ctx);   // captured sweeps hold pointers into the old workspace
     return FR_OK;
 }
 
-// After a failed or abandoned queue sweep: BFS marks, corridor bits and block sides idle.
-fr_status reset_queue_idle(fr_ctx *ctx) {
+// After a failed or abandoned launch: BFS marks, corridor bits and block sides idle.
+fr_status reset_queue_idle(fr_ctx *ctx, QueueMem &Q) {
     fr_status st = reset_idle(ctx);
     if (st != FR_OK) return st;
-    const QCaps c = caps_for(ctx->q_ctas, ctx->q_n);
-    for (const QSlot &S : ctx->q_host) {
-        CK(cudaMemsetAsync(S.sob, 0xFF, sizeof(int) * (size_t)ctx->q_k, ctx->stream));
+    const QCaps c = caps_for(Q.ctas, Q.n);
+    for (const QSlot &S : Q.host) {
+        CK(cudaMemsetAsync(S.sob, 0xFF, sizeof(int) * (size_t)Q.k, ctx->stream));
         CK(cudaMemsetAsync(S.cbits, 0, sizeof(unsigned int) * (size_t)c.words, ctx->stream));
         CK(cudaMemsetAsync(S.sdbits, 0, sizeof(unsigned int) * (size_t)c.words, ctx->stream));
         CK(cudaMemsetAsync(S.sbits, 0, sizeof(unsigned int) * (size_t)c.swords, ctx->stream));
@@ -213,16 +232,9 @@ fr_status reset_queue_idle(fr_ctx *ctx) {
 
 }  // namespace
 
-void free_queue(fr_ctx *ctx) {
-    if (ctx->q_mem) cudaFree(ctx->q_mem);
-    ctx->q_mem = nullptr;
-    ctx->q_bytes = 0;
-    ctx->q_ctas = ctx->q_clusters = ctx->q_n = ctx->q_nnz = ctx->q_k = ctx->q_reps = ctx->q_np = 0;
-    ctx->q_host.clear();
-    ctx->q_slots = nullptr;
-    ctx->q_graphs = nullptr;
-    ctx->q_ctls = nullptr;
-    ctx->q_stats = nullptr;
+void free_queue(QueueMem &Q) {
+    if (Q.mem) cudaFree(Q.mem);
+    Q = QueueMem();
 }
 
 int queue_size_for(fr_ctx *ctx, const BatchPlan &pl, const fr_options *opt) {
@@ -255,7 +267,7 @@ int queue_size_for(fr_ctx *ctx, const BatchPlan &pl, const fr_options *opt) {
                          std::sqrt(chain * chain + turns * turns) *
                              (est <= kTiny ? kRelTiny : est <= kSmall ? kRelSmall : kRelTime)[t];
         if (best < 0 || v < bestv) { best = t; bestv = v; }
-        if (ctx->q_mem && ctx->q_ctas == c) { kept = t; keptv = v; }
+        if (ctx->sweep_q.mem && ctx->sweep_q.ctas == c) { kept = t; keptv = v; }
     }
     // The size laid out already, unless another is clearly better: laying out again takes a few
     // tenths of a millisecond and drops the captured sweeps (a V-cycle of grid3d 108,570
@@ -272,7 +284,8 @@ fr_status run_queue_sweep(fr_ctx *ctx, const fr_graph *g, int32_t *part, const B
     int clusters = std::max(1, std::min(ctx->q_cap[t], pl.np));
     if (opt->grid_blocks > 0) clusters = std::max(1, std::min(clusters, opt->grid_blocks / ctas));
     const int reps = opt->mb_reps > 0 ? opt->mb_reps : 1;
-    fr_status st = ensure_queue(ctx, ctas, clusters, g->n, g->nnz, pl.k, reps, pl.np);
+    QueueMem &Q = ctx->sweep_q;
+    fr_status st = ensure_queue(ctx, Q, ctas, clusters, g->n, g->nnz, pl.k, reps, pl.np);
     if (st != FR_OK) return st;
     // per-cluster graph descriptors (each with its own sob) and each pair's predecessors
     GraphDev *hg = reinterpret_cast<GraphDev *>(ctx->h_stage + kStageGraphs);
@@ -281,7 +294,7 @@ fr_status run_queue_sweep(fr_ctx *ctx, const fr_graph *g, int32_t *part, const B
         memset(&gd, 0, sizeof(gd));
         gd.xadj = g->xadj; gd.adjncy = g->adjncy; gd.adjwgt = g->adjwgt; gd.vwgt = g->vwgt;
         gd.part = part; gd.dist = ctx->dist; gd.lid = ctx->lid;
-        gd.sob = ctx->q_host[i].sob;
+        gd.sob = Q.host[i].sob;
         gd.blockw = ctx->blockw;
         gd.n = g->n; gd.nnz = g->nnz; gd.k = pl.k; gd.base = 0; gd.Lmax = pl.Lmax;
         gd.bl = ctx->bl; gd.blc = ctx->blc; gd.inb = ctx->inb;
@@ -295,41 +308,41 @@ fr_status run_queue_sweep(fr_ctx *ctx, const fr_graph *g, int32_t *part, const B
             last[pl.pa[j]] = last[pl.pb[j]] = j;
         }
     }
-    CK(cudaMemcpyAsync(ctx->q_graphs, hg, sizeof(GraphDev) * (size_t)clusters, cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaMemcpyAsync(ctx->q_prev, hp, sizeof(int) * 2 * (size_t)pl.np, cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaMemcpyAsync(Q.graphs, hg, sizeof(GraphDev) * (size_t)clusters, cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaMemcpyAsync(Q.prev, hp, sizeof(int) * 2 * (size_t)pl.np, cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(ctx->part_backup, part, sizeof(int) * (size_t)g->n, cudaMemcpyDeviceToDevice, ctx->stream));
 
     QueueArgs q;
     memset(&q, 0, sizeof(q));
     q.wt = make_work(ctx, 0, 0, pl.np, g->n, opt);
-    q.wt.vq_cap = (int)ctx->q_vq;
-    q.wt.nu_cap = (int)ctx->q_nu;
-    q.wt.mu_cap = (int)ctx->q_mu;
-    q.wt.crank = ctx->q_crank;
+    q.wt.vq_cap = (int)Q.vq;
+    q.wt.nu_cap = (int)Q.nu;
+    q.wt.mu_cap = (int)Q.mu;
+    q.wt.crank = Q.crank;
     q.wt.total_n = g->n;
-    q.wt.qb_sorted = ctx->qb_sorted;
-    q.wt.qb_start = ctx->qb_start;
-    q.wt.qb_app = ctx->qb_app;
-    q.wt.qb_pool = ctx->qb_pool;
-    q.wt.qb_lst = ctx->qb_lst;
-    q.wt.qb_cap = ctx->qb_cap;
-    q.slots = ctx->q_slots;
+    q.wt.qb_sorted = Q.qb_sorted;
+    q.wt.qb_start = Q.qb_start;
+    q.wt.qb_app = Q.qb_app;
+    q.wt.qb_pool = Q.qb_pool;
+    q.wt.qb_lst = Q.qb_lst;
+    q.wt.qb_cap = Q.qb_cap;
+    q.slots = Q.slots;
     q.np = pl.np;
-    q.ticket = ctx->q_ticket;
-    q.votes = q.wt.flow_sched == 0 ? ctx->q_ticket + 1 : nullptr;
-    q.prev = ctx->q_prev;
-    q.gabort = ctx->q_gabort;
+    q.ticket = Q.ticket;
+    q.votes = q.wt.flow_sched == 0 ? Q.ticket + 1 : nullptr;
+    q.prev = Q.prev;
+    q.gabort = Q.gabort;
     q.wait_ns = kWaitNs;
 
     auto enqueue = [&]() -> fr_status {
         CK(launch_fill_pairs(ctx->pairs, ctx->pair_a, ctx->pair_b, pl.np, 0, opt->mb ? 1 : 0, pl.Ubase, ctx->stream));
         CK(cudaMemsetAsync(ctx->sides, 0, sizeof(SideDev) * 2 * (size_t)pl.np, ctx->stream));
         CK(cudaMemsetAsync(ctx->pacc, 0, sizeof(PairAcc) * (size_t)pl.np, ctx->stream));
-        CK(cudaMemsetAsync(ctx->q_ticket, 0, queue_state_bytes(ctx, clusters), ctx->stream));
-        CK(cudaMemsetAsync(ctx->qb_lst, 0xFF, sizeof(int) * (size_t)g->n, ctx->stream));
-        CK(cudaMemsetAsync(ctx->qb_cnt, 0, sizeof(int) * (size_t)pl.k, ctx->stream));
-        CK(launch_qb_build(ctx->bl, ctx->blc, part, pl.k, ctx->qb_cnt, ctx->qb_start, ctx->qb_app, ctx->qb_lst,
-                           ctx->qb_sorted, ctx->stream));
+        CK(cudaMemsetAsync(Q.ticket, 0, queue_state_bytes(Q, clusters), ctx->stream));
+        CK(cudaMemsetAsync(Q.qb_lst, 0xFF, sizeof(int) * (size_t)g->n, ctx->stream));
+        CK(cudaMemsetAsync(Q.qb_cnt, 0, sizeof(int) * (size_t)pl.k, ctx->stream));
+        CK(launch_qb_build(ctx->bl, ctx->blc, part, pl.k, Q.qb_cnt, Q.qb_start, Q.qb_app, Q.qb_lst,
+                           Q.qb_sorted, ctx->stream));
         if (ctx->profiling) CK(cudaEventRecord(ctx->pev[0], ctx->stream));
         CK(launch_queue_sweep(q, ctas, clusters, ctx->stream));
         if (ctx->profiling) CK(cudaEventRecord(ctx->pev[1], ctx->stream));
@@ -346,7 +359,7 @@ fr_status run_queue_sweep(fr_ctx *ctx, const fr_graph *g, int32_t *part, const B
     std::vector<long long> key = {-7, (long long)(uintptr_t)g->xadj, (long long)(uintptr_t)part, g->n, g->nnz,
                                   pl.np, pl.Ubase, opt->mb, reps, (long long)opt->seed, opt->gr_interval,
                                   opt->inner_ops, opt->pulse_cap, (long long)(uintptr_t)ctx->base_mem,
-                                  (long long)(uintptr_t)ctx->pair_mem, (long long)(uintptr_t)ctx->q_mem,
+                                  (long long)(uintptr_t)ctx->pair_mem, (long long)(uintptr_t)Q.mem,
                                   ctx->tune_gr, ctx->tune_inner, opt->pulse_passes, ctx->tune_passes,
                                   opt->flow_sched, ctx->tune_sched, ctx->narrow_ok, opt->pre_waves,
                                   ctx->tune_prewaves, ctas, clusters, pl.Lmax, opt->gap_interval};
@@ -397,9 +410,9 @@ fr_status run_queue_sweep(fr_ctx *ctx, const fr_graph *g, int32_t *part, const B
     ctx->sweep_launches = launches;
     ctx->last_launches = launches;
     int gab = 0;
-    CK(cudaMemcpyAsync(&gab, ctx->q_gabort, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-    std::vector<fr_ctx::QCtl> qc(clusters);
-    CK(cudaMemcpyAsync(qc.data(), ctx->q_ctls, sizeof(fr_ctx::QCtl) * (size_t)clusters, cudaMemcpyDeviceToHost,
+    CK(cudaMemcpyAsync(&gab, Q.gabort, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    std::vector<QueueMem::QCtl> qc(clusters);
+    CK(cudaMemcpyAsync(qc.data(), Q.ctls, sizeof(QueueMem::QCtl) * (size_t)clusters, cudaMemcpyDeviceToHost,
                        ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     ctls->resize(clusters);
@@ -409,7 +422,7 @@ fr_status run_queue_sweep(fr_ctx *ctx, const fr_graph *g, int32_t *part, const B
     if (gab != 0) {
         // leave part exactly as it was, and the workspace idle
         CK(cudaMemcpyAsync(part, ctx->part_backup, sizeof(int) * (size_t)g->n, cudaMemcpyDeviceToDevice, ctx->stream));
-        if ((st = reset_queue_idle(ctx)) != FR_OK) return st;
+        if ((st = reset_queue_idle(ctx, Q)) != FR_OK) return st;
         if (gab == E_MISFIT) {
             ++ctx->queue_fallbacks;
             int where = 0;
@@ -481,7 +494,7 @@ int queue_round_size(fr_ctx *ctx, int P, long long est, double avg_degree, const
         const double v = est <= kTiny ? (double)c :
                                         (double)((P + ctx->q_cap[t] - 1) / ctx->q_cap[t]) * kRelTime[t];
         if (best < 0 || v < bestc) { best = t; bestc = v; }
-        if (ctx->q_mem && ctx->q_ctas == c) { kept = t; keptc = v; }
+        if (ctx->round_q.mem && ctx->round_q.ctas == c) { kept = t; keptc = v; }
     }
     // the size laid out already, unless another is clearly better
     return kept >= 0 && keptc <= 1.25 * bestc ? kept : best;
@@ -494,7 +507,8 @@ fr_status enqueue_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int
     int clusters = std::max(1, std::min(ctx->q_cap[t], P));
     if (opt->grid_blocks > 0) clusters = std::max(1, std::min(clusters, opt->grid_blocks / ctas));
     const int reps = opt->mb_reps > 0 ? opt->mb_reps : 1;
-    const fr_status st = ensure_queue(ctx, ctas, clusters, g->n, g->nnz, k, reps, P);
+    QueueMem &Q = ctx->round_q;
+    const fr_status st = ensure_queue(ctx, Q, ctas, clusters, g->n, g->nnz, k, reps, P);
     if (st == FR_ERR_OOM) return FR_OK;   // no room under the arena bound: the round's own launches
     if (st != FR_OK) return st;
     GraphDev *hg = reinterpret_cast<GraphDev *>(ctx->h_stage + kStageRound);
@@ -505,12 +519,12 @@ fr_status enqueue_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int
         memset(&gd, 0, sizeof(gd));
         gd.xadj = g->xadj; gd.adjncy = g->adjncy; gd.adjwgt = g->adjwgt; gd.vwgt = g->vwgt;
         gd.part = part; gd.dist = ctx->dist; gd.lid = ctx->lid;
-        gd.sob = ctx->q_host[i].sob;
+        gd.sob = Q.host[i].sob;
         gd.blockw = ctx->blockw;
         gd.n = g->n; gd.nnz = g->nnz; gd.k = k; gd.base = 0; gd.Lmax = Lmax;
         gd.bl = ctx->bl; gd.blc = ctx->blc; gd.inb = ctx->inb;
     }
-    CK(cudaMemcpyAsync(ctx->q_graphs, hg, sizeof(GraphDev) * (size_t)clusters, cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaMemcpyAsync(Q.graphs, hg, sizeof(GraphDev) * (size_t)clusters, cudaMemcpyHostToDevice, ctx->stream));
     // part and the block weights as they are, should a pair outgrow its cluster
     CK(cudaMemcpyAsync(ctx->spare, part, sizeof(int) * (size_t)g->n, cudaMemcpyDeviceToDevice, ctx->stream));
     CK(cudaMemcpyAsync(ctx->h_stage + kStageRoundW, ctx->blockw, sizeof(long long) * (size_t)k, cudaMemcpyDeviceToHost,
@@ -518,25 +532,25 @@ fr_status enqueue_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int
     QueueArgs q;
     memset(&q, 0, sizeof(q));
     q.wt = make_work(ctx, 0, 0, P, g->n, opt);
-    q.wt.vq_cap = (int)ctx->q_vq;
-    q.wt.nu_cap = (int)ctx->q_nu;
-    q.wt.mu_cap = (int)ctx->q_mu;
-    q.wt.crank = ctx->q_crank;
+    q.wt.vq_cap = (int)Q.vq;
+    q.wt.nu_cap = (int)Q.nu;
+    q.wt.mu_cap = (int)Q.mu;
+    q.wt.crank = Q.crank;
     q.wt.total_n = g->n;
-    q.slots = ctx->q_slots;
+    q.slots = Q.slots;
     q.np = P;
-    q.ticket = ctx->q_ticket;
+    q.ticket = Q.ticket;
     q.prev = nullptr;   // no pair waits for another
-    q.gabort = ctx->q_gabort;
+    q.gabort = Q.gabort;
     q.wait_ns = kWaitNs;
-    CK(cudaMemsetAsync(ctx->q_ticket, 0, queue_state_bytes(ctx, clusters), ctx->stream));
+    CK(cudaMemsetAsync(Q.ticket, 0, queue_state_bytes(Q, clusters), ctx->stream));
     if (P > 1) {   // pairs commit to the list while others scan it: they scan what is on it now
-        q.wt.scan_len = ctx->q_ticket + 2;
-        CK(cudaMemcpyAsync(ctx->q_ticket + 2, ctx->blc, sizeof(int), cudaMemcpyDeviceToDevice, ctx->stream));
+        q.wt.scan_len = Q.ticket + 2;
+        CK(cudaMemcpyAsync(Q.ticket + 2, ctx->blc, sizeof(int), cudaMemcpyDeviceToDevice, ctx->stream));
     }
     CK(launch_queue_sweep(q, ctas, clusters, ctx->stream));
     char *h = ctx->h_stage + kStageRoundCtl;
-    CK(cudaMemcpyAsync(h, ctx->q_gabort, 256 + sizeof(fr_ctx::QCtl) * (size_t)clusters, cudaMemcpyDeviceToHost,
+    CK(cudaMemcpyAsync(h, Q.gabort, 256 + sizeof(QueueMem::QCtl) * (size_t)clusters, cudaMemcpyDeviceToHost,
                        ctx->stream));
     rq->queued = true;
     rq->clusters = clusters;
@@ -546,7 +560,7 @@ fr_status enqueue_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int
 fr_status finish_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int k, const char *where, RoundQueue *rq) {
     const char *h = ctx->h_stage + kStageRoundCtl;
     const int gab = *reinterpret_cast<const int *>(h);
-    const fr_ctx::QCtl *qc = reinterpret_cast<const fr_ctx::QCtl *>(h + 256);
+    const QueueMem::QCtl *qc = reinterpret_cast<const QueueMem::QCtl *>(h + 256);
     memset(&rq->ctl, 0, sizeof(rq->ctl));
     for (int i = 0; i < rq->clusters; ++i) {
         const Ctl &c = qc[i].c;
@@ -560,7 +574,7 @@ fr_status finish_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int 
         }
     }
     if (gab == 0) return FR_OK;
-    fr_status st = reset_queue_idle(ctx);
+    fr_status st = reset_queue_idle(ctx, ctx->round_q);
     if (st != FR_OK) return st;
     if (gab == E_MISFIT) {
         rq->queued = false;
