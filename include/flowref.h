@@ -201,13 +201,18 @@ int32_t fr_struct_size(int32_t which);
 
 /* Creates a context on `device` using `stream` (a cudaStream_t; NULL = a new
  * non-blocking stream owned by the context).  arena_bytes bounds the device
- * workspace (0 = no bound); exceeding it returns FR_ERR_OOM. */
+ * workspace (0 = no bound); exceeding it returns FR_ERR_OOM.  Under a bound a call
+ * gives back workspaces of earlier calls that it does without before it exceeds it,
+ * and the queue workspace of single rounds is taken only where it fits.  (The FM and
+ * multi-try state is admitted by its size beside the graph and pair arrays; the sweep
+ * arrays of the same call, 20 bytes a vertex and sweep, are not added to that.) */
 fr_status fr_create(fr_ctx **ctx, int32_t device, size_t arena_bytes, void *stream);
 fr_status fr_destroy(fr_ctx *ctx);
 /* Message of the last failing call on this context (static storage in ctx). */
 const char *fr_last_error(const fr_ctx *ctx);
 const char *fr_status_string(fr_status st);
-/* Bytes of device workspace the context holds now. */
+/* Bytes of device workspace the context holds now (the device copy that
+ * fr_refine_batch_host makes of its graph is not workspace). */
 size_t fr_workspace_bytes(const fr_ctx *ctx);
 
 /* ---- the three steps of Section 4.1 on one pair --------------------------- */

@@ -138,6 +138,31 @@ static size_t reps_bytes(long long nu, long long P, int reps) {
     return b;
 }
 
+size_t held_bytes(const fr_ctx *ctx) {
+    return ctx->base_bytes + ctx->pair_bytes + ctx->reps_bytes + ctx->fm_bytes + ctx->mt_bytes + ctx->sweep_q.bytes +
+           ctx->round_q.bytes;
+}
+
+static bool give_back(fr_ctx *ctx) {
+    if (ctx->round_q.mem) free_queue(ctx->round_q);
+    else if (ctx->sweep_q.mem) free_queue(ctx->sweep_q);
+    else if (ctx->fm_mem && !ctx->fm_live) free_fm(ctx);
+    else if (ctx->mt_mem && !ctx->mt_live) free_mt(ctx);
+    else return false;
+    return true;
+}
+
+cudaError_t alloc_workspace(fr_ctx *ctx, void **mem, size_t bytes) {
+    while (ctx->arena_limit && held_bytes(ctx) + bytes > ctx->arena_limit && give_back(ctx)) {}
+    cudaError_t e;
+    while ((e = cudaMalloc(mem, bytes)) != cudaSuccess) {
+        cudaGetLastError();
+        *mem = nullptr;
+        if (!give_back(ctx)) break;
+    }
+    return e;
+}
+
 fr_status ensure_reps(fr_ctx *ctx, int reps) {
     if (reps < 1) reps = 1;
     const long long nu = ctx->n_cap;
@@ -153,8 +178,7 @@ fr_status ensure_reps(fr_ctx *ctx, int reps) {
     if (ctx->reps_mem) cudaFree(ctx->reps_mem);
     ctx->reps_mem = nullptr;
     ctx->reps_bytes = 0;
-    if (cudaMalloc(&ctx->reps_mem, bytes) != cudaSuccess) {
-        cudaGetLastError();
+    if (alloc_workspace(ctx, &ctx->reps_mem, bytes) != cudaSuccess) {
         ctx_error(ctx, "cudaMalloc(%zu) for sweep state failed", bytes);
         return FR_ERR_OOM;
     }
@@ -188,6 +212,7 @@ static void free_pairs(fr_ctx *ctx) {
 
 fr_status ensure_base(fr_ctx *ctx, int n, int nnz, int k, int reps) {
     if (reps < 1) reps = 1;
+    ctx->fm_live = ctx->mt_live = false;   // (every call comes here first)
     if (ctx->base_mem && n <= ctx->n_cap && nnz <= ctx->nnz_cap && k <= ctx->k_cap)
         return ensure_reps(ctx, reps);
     const int nn = std::max(n, ctx->n_cap), mm = std::max(nnz, ctx->nnz_cap);
@@ -199,10 +224,8 @@ fr_status ensure_base(fr_ctx *ctx, int n, int nnz, int k, int reps) {
         return FR_ERR_OOM;
     }
     free_base(ctx);
-    cudaError_t e = cudaMalloc(&ctx->base_mem, bytes);
+    cudaError_t e = alloc_workspace(ctx, &ctx->base_mem, bytes);
     if (e != cudaSuccess) {
-        ctx->base_mem = nullptr;
-        cudaGetLastError();
         ctx_error(ctx, "cudaMalloc(%zu) for the workspace failed: %s", bytes, cudaGetErrorString(e));
         return FR_ERR_OOM;
     }
@@ -249,6 +272,7 @@ fr_status ensure_base(fr_ctx *ctx, int n, int nnz, int k, int reps) {
 }
 
 fr_status ensure_fm(fr_ctx *ctx, int n, int nnz, int k, int P) {
+    ctx->fm_live = true;
     if (ctx->fm_mem && n <= ctx->fm_n && nnz <= ctx->fm_nnz && k <= ctx->fm_k && P <= ctx->fm_p) return FR_OK;
     const long long nn = std::max(n, ctx->fm_n), mm = std::max(nnz, ctx->fm_nnz);
     const int kk = std::max(k, ctx->fm_k), pp = std::max(P, ctx->fm_p);
@@ -267,9 +291,7 @@ fr_status ensure_fm(fr_ctx *ctx, int n, int nnz, int k, int P) {
         return FR_ERR_OOM;
     }
     free_fm(ctx);
-    if (cudaMalloc(&ctx->fm_mem, b) != cudaSuccess) {
-        ctx->fm_mem = nullptr;
-        cudaGetLastError();
+    if (alloc_workspace(ctx, &ctx->fm_mem, b) != cudaSuccess) {
         ctx_error(ctx, "cudaMalloc(%zu) for the FM workspace failed", b);
         return FR_ERR_OOM;
     }
@@ -320,10 +342,8 @@ fr_status ensure_pairs(fr_ctx *ctx, int P, int R, int reps) {
         return FR_ERR_OOM;
     }
     free_pairs(ctx);
-    cudaError_t e = cudaMalloc(&ctx->pair_mem, bytes);
+    cudaError_t e = alloc_workspace(ctx, &ctx->pair_mem, bytes);
     if (e != cudaSuccess) {
-        ctx->pair_mem = nullptr;
-        cudaGetLastError();
         ctx_error(ctx, "cudaMalloc(%zu) for pair state failed", bytes);
         return FR_ERR_OOM;
     }
@@ -528,7 +548,7 @@ extern "C" const char *fr_status_string(fr_status st) {
 }
 
 extern "C" size_t fr_workspace_bytes(const fr_ctx *ctx) {
-    return ctx ? ctx->base_bytes + ctx->pair_bytes + ctx->reps_bytes : 0;
+    return ctx ? held_bytes(ctx) : 0;
 }
 
 // ---------------------------------------------------------- argument checks --

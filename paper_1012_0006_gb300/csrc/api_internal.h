@@ -140,6 +140,7 @@ struct fr_ctx {
     // its launches: one for sweeps, one for single rounds (pairs, active scheduling)
     int q_cap[kNumClusterSizes] = {0, 0, 0, 0, 0};
     QueueMem sweep_q, round_q;
+    bool fm_live = false, mt_live = false;     // the running call uses the FM / multi-try workspace
     bool last_queue = false;                   // the last fr_refine_batch ran as a queue sweep
     int last_queue_ctas = 0, last_queue_clusters = 0, queue_fallbacks = 0;
 };
@@ -170,6 +171,13 @@ fr_status cuda_fail(fr_ctx *ctx, cudaError_t e, const char *what);
 long long host_budget_base(long long W, int k, double eps, double alpha);
 long long host_lmax(long long W, long long maxc, int k, double eps);
 fr_status status_from_ctl(fr_ctx *ctx, const fr::Ctl &c, const char *where);
+// Bytes of every workspace the context holds.
+size_t held_bytes(const fr_ctx *ctx);
+// Device memory for a workspace that the running call needs and its bound admits.  While what
+// is held with it exceeds the bound, or the device has no room, workspaces that the call does
+// without are given back: the queue kernel's (laid out again when one is used), then the FM and
+// multi-try state of earlier calls.
+cudaError_t alloc_workspace(fr_ctx *ctx, void **mem, size_t bytes);
 fr_status ensure_base(fr_ctx *ctx, int n, int nnz, int k, int reps);
 fr_status ensure_pairs(fr_ctx *ctx, int P, int R, int reps);
 fr_status ensure_reps(fr_ctx *ctx, int reps);

@@ -31,6 +31,7 @@ T *carve_mt(char *&p, long long count) {
 }  // namespace
 
 fr_status ensure_mt(fr_ctx *ctx, int n, int nnz, int k, int P) {
+    ctx->mt_live = true;
     if (ctx->mt_mem && n <= ctx->mt_n && nnz <= ctx->mt_nnz && k <= ctx->mt_k && P <= ctx->mt_p) return FR_OK;
     const long long nn = std::max(n, ctx->mt_n), mm = std::max(nnz, ctx->mt_nnz);
     const int kk = std::max(k, ctx->mt_k), pp = std::max(P, ctx->mt_p);
@@ -59,9 +60,7 @@ fr_status ensure_mt(fr_ctx *ctx, int n, int nnz, int k, int P) {
         return FR_ERR_OOM;
     }
     free_mt(ctx);
-    if (cudaMalloc(&ctx->mt_mem, b) != cudaSuccess) {
-        ctx->mt_mem = nullptr;
-        cudaGetLastError();
+    if (alloc_workspace(ctx, &ctx->mt_mem, b) != cudaSuccess) {
         ctx_error(ctx, "cudaMalloc(%zu) for the multi-try workspace failed", b);
         return FR_ERR_OOM;
     }

@@ -132,20 +132,19 @@ fr_status ensure_queue(fr_ctx *ctx, QueueMem &Q, int ctas, int clusters, int n, 
     const int rr = std::max(reps, same ? Q.reps : 1), pp = std::max(np, same ? Q.np : 0);
     const int cc = std::max(clusters, same ? Q.clusters : 0);
     const size_t bytes = queue_bytes(ctas, cc, nn, mm, kk, rr, pp, sweep);
-    // A round's workspace is taken where it fits beside the sweeps' (its launches have another
-    // form), and makes room for theirs.
-    const size_t others = ctx->base_bytes + ctx->pair_bytes + ctx->reps_bytes + (sweep ? 0 : ctx->sweep_q.bytes);
+    // A round's workspace is taken where it fits beside everything held (its launches have
+    // another form); the sweeps' is needed, and others make room for it.
+    const size_t others = sweep ? ctx->base_bytes + ctx->pair_bytes + ctx->reps_bytes : held_bytes(ctx) - Q.bytes;
     if (ctx->arena_limit && bytes + others > ctx->arena_limit) {
         ctx_error(ctx, "queue sweep workspace exceeds the arena bound");
         return FR_ERR_OOM;
     }
-    if (sweep && ctx->arena_limit && bytes + others + ctx->round_q.bytes > ctx->arena_limit) free_queue(ctx->round_q);
     // Another cluster size lays the same memory out again where it is large enough: a V-cycle
     // and the rounds of active scheduling change sizes often, and a cudaFree and cudaMalloc
     // pair takes longer than a small round.
     if (!Q.mem || bytes > Q.bytes) {
         free_queue(Q);
-        if (cudaMalloc(&Q.mem, bytes) != cudaSuccess) {
+        if ((sweep ? alloc_workspace(ctx, &Q.mem, bytes) : cudaMalloc(&Q.mem, bytes)) != cudaSuccess) {
             cudaGetLastError();
             Q.mem = nullptr;
             ctx_error(ctx, "cudaMalloc(%zu) for the queue sweep failed", bytes);

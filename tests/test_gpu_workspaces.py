@@ -43,3 +43,66 @@ def test_a_pair_call_leaves_room_for_a_sweep(gpu_lib, ctas):
     assert len({s for v in admitted.values() for s in v}) > 1   # the bounds reach from refused to admitted
     for mib, (own, queue) in admitted.items():
         assert own == queue, mib
+
+
+def _calls(F, c, w, sched, check=False):
+    """Pairs and active scheduling with FM and multi-try, sweeps and k-way rounds in turn on one context;
+    after each: its status, what the context holds, the partition."""
+    k, out = w["k"], []
+    for call in ("pair", "active", "batch", "fm", "kway", "pair", "batch", "active"):
+        g, part = _dev(F, w)
+        fm = dict(mb=1, fm_permille=50)
+        if call == "pair":
+            st, *_ = c.refine_pair(g, part, k, 0, 1, w["eps"], w["alpha"], F.default_options(**fm, sweep_sched=sched),
+                                   check=check)
+        elif call == "active":
+            st, *_ = c.refine_active(g, part, k, w["eps"], w["alpha"],
+                                     F.default_options(**fm, mt_alpha=10, sweep_sched=sched), max_outer=1, check=check)
+        elif call == "batch":
+            st, *_ = c.refine_batch(g, part, k, w["eps"], w["alpha"], F.default_options(mb=1, mb_reps=2), check=check)
+        elif call == "fm":
+            st, *_ = c.refine_batch(g, part, k, w["eps"], w["alpha"], F.default_options(**fm), check=check)
+        else:
+            st, _ = c.kway_global(g, part, k, w["eps"], init_mode=0, alpha=10, max_rounds=1, seed=1, check=check)
+        out.append((st, c.workspace_bytes, part.cpu().numpy()))
+    return out
+
+
+def test_a_bounded_context_stays_within_its_bound(gpu_lib):
+    F = gpu_lib
+    w = _grid(160, 150, 8)
+    with F.Context(0) as c:
+        want = _calls(F, c, w, 1, check=True)
+    start = np.array(w["part"], np.int32)
+    seen = set()
+    for mib in range(4, 420, 8):
+        bound = mib << 20
+        with F.Context(0, arena_bytes=bound) as c:
+            own = _calls(F, c, w, 1)
+        with F.Context(0, arena_bytes=bound) as c:
+            queue = _calls(F, c, w, 0)
+        for i in range(len(want)):
+            assert queue[i][0] == own[i][0], (mib, i)   # admitted as with the round's own launches
+            # (what those hold: the sweep arrays of an FM call are not added to its bound)
+            assert queue[i][1] <= max(bound, own[i][1]), (mib, i)
+            assert np.array_equal(queue[i][2], want[i][2] if queue[i][0] == 0 else start), (mib, i)
+            seen.add(queue[i][0])
+    assert seen == {0, F.FR_ERR_OOM}
+
+
+def test_workspace_bytes_counts_what_is_held(gpu_lib):
+    import torch
+    F = gpu_lib
+    w = _grid(700, 600, 8)
+    with F.Context(0) as c:   # (kernels and contexts loaded before the count)
+        _calls(F, c, w, 0, check=True)
+    _, part = _dev(F, w)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    before = torch.cuda.mem_get_info()[0]
+    with F.Context(0) as c:
+        _calls(F, c, w, 0, check=True)
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        used, held = before - torch.cuda.mem_get_info()[0], c.workspace_bytes
+    assert abs(used - held) < 32 << 20   # (device memory comes in blocks of 2 MiB)
