@@ -127,15 +127,21 @@ fr_status ensure_queue(fr_ctx *ctx, QueueMem &Q, int ctas, int clusters, int n, 
         np <= Q.np)
         return FR_OK;
     const bool sweep = &Q == &ctx->sweep_q;
-    const bool same = Q.ctas == ctas;
-    const int nn = std::max(n, same ? Q.n : 0), mm = std::max(nnz, same ? Q.nnz : 0), kk = std::max(k, same ? Q.k : 0);
-    const int rr = std::max(reps, same ? Q.reps : 1), pp = std::max(np, same ? Q.np : 0);
-    const int cc = std::max(clusters, same ? Q.clusters : 0);
-    const size_t bytes = queue_bytes(ctas, cc, nn, mm, kk, rr, pp, sweep);
+    int nn = n, mm = nnz, kk = k, rr = std::max(reps, 1), pp = np, cc = clusters;
+    if (Q.ctas == ctas) {   // as large as the calls before asked for
+        nn = std::max(nn, Q.n); mm = std::max(mm, Q.nnz); kk = std::max(kk, Q.k);
+        rr = std::max(rr, Q.reps); pp = std::max(pp, Q.np); cc = std::max(cc, Q.clusters);
+    }
     // A round's workspace is taken where it fits beside everything held (its launches have
     // another form); the sweeps' is needed, and others make room for it.
     const size_t others = sweep ? ctx->base_bytes + ctx->pair_bytes + ctx->reps_bytes : held_bytes(ctx) - Q.bytes;
-    if (ctx->arena_limit && bytes + others > ctx->arena_limit) {
+    auto fits = [&](size_t b) { return ctx->arena_limit == 0 || b + others <= ctx->arena_limit; };
+    size_t bytes = queue_bytes(ctas, cc, nn, mm, kk, rr, pp, sweep);
+    if (!fits(bytes)) {   // what this call asks for alone
+        nn = n; mm = nnz; kk = k; rr = std::max(reps, 1); pp = np; cc = clusters;
+        bytes = queue_bytes(ctas, cc, nn, mm, kk, rr, pp, sweep);
+    }
+    if (!fits(bytes)) {
         ctx_error(ctx, "queue sweep workspace exceeds the arena bound");
         return FR_ERR_OOM;
     }

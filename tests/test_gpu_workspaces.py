@@ -106,3 +106,33 @@ def test_workspace_bytes_counts_what_is_held(gpu_lib):
         torch.cuda.empty_cache()
         used, held = before - torch.cuda.mem_get_info()[0], c.workspace_bytes
     assert abs(used - held) < 32 << 20   # (device memory comes in blocks of 2 MiB)
+
+
+def test_a_sweep_of_other_sizes_is_admitted_alone(gpu_lib):
+    """A graph with many vertices and few pairs, then one with few vertices and many pairs: under
+    a bound that holds the workspace of each, not one of both sizes together."""
+    F = gpu_lib
+    large, small = _grid(320, 300, 2), _grid(64, 61, 16)
+    opts = F.default_options(mb=1, cluster_ctas=4)
+    st, pref, _, _ = O.refine_batch(small, opts=O.options(mb=1))
+    assert st == 0
+
+    def sweep(c, w):
+        g, part = _dev(F, w)
+        st, *_ = c.refine_batch(g, part, w["k"], w["eps"], w["alpha"], opts, check=False)
+        return st, part.cpu().numpy()
+
+    seen = set()
+    for mib in range(40, 240, 4):
+        with F.Context(0, arena_bytes=mib << 20) as c:   # the large graph's arrays, no queue workspace of its
+            g, part = _dev(F, large)
+            c.refine_batch(g, part, 2, large["eps"], large["alpha"], F.default_options(mb=1, sweep_sched=1))
+            alone = sweep(c, small)
+        with F.Context(0, arena_bytes=mib << 20) as c:
+            assert sweep(c, large)[0] == 0
+            after = sweep(c, small)
+            assert c.workspace_bytes <= mib << 20
+        assert after[0] == alone[0], mib
+        assert np.array_equal(after[1], pref if after[0] == 0 else np.array(small["part"], np.int32))
+        seen.add(after[0])
+    assert seen == {0, F.FR_ERR_OOM}
