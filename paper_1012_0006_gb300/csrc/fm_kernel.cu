@@ -184,7 +184,7 @@ __device__ __forceinline__ void fm_ahead(const GraphDev &G, const FmDev &f, FmSh
     unsigned acc = 0;
     auto warm = [&](int v, int j0, int j1) {
         acc ^= (unsigned)__ldg(G.vwgt + v);
-        for (int j = j0 + lane; j < min(j1, nnz); j += 32)
+        for (int j = j0 + lane, end = fm_row_end(j0, j1, nnz); j < end; j += 32)
             acc ^= (unsigned)__ldg(G.adjwgt + j) ^ (unsigned)f.rec[__ldg(G.adjncy + j)].x;
     };
     int seed = me, push = me;

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include "fm_limits.h"
 #include "fr_internal.cuh"
 
 namespace fr {
@@ -37,10 +38,9 @@ struct FmDev {
     int permille;
 };
 
-// Ten bits each in a record: |gain| <= weighted degree < 1024, and arc weights are at least 1.
-__host__ __device__ constexpr int fm_in(int x) { return x & 1023; }
-__host__ __device__ constexpr int fm_ext(int x) { return (x >> 10) & 1023; }
-__host__ __device__ constexpr int fm_deg(int x) { return (x >> 20) & 1023; }
+__host__ __device__ constexpr int fm_in(int x) { return x & kFmMaxDeg; }
+__host__ __device__ constexpr int fm_ext(int x) { return (x >> 10) & kFmMaxDeg; }
+__host__ __device__ constexpr int fm_deg(int x) { return (x >> 20) & kFmMaxDeg; }
 
 // Enqueues the FM searches of the round described by w (one graph with k blocks,
 // w.npairs pairs): block counts, pair regions, boundary gather, one CTA per pair.
