@@ -93,7 +93,8 @@ typedef struct fr_options {
                               vertices moved without an improvement (50 = the 5 % of the
                               paper's setup); 0 = no FM.  fr_refine_pair, fr_refine_batch and
                               fr_refine_active; needs a simple graph and every gain within
-                              +-1023 (max weighted degree of the graph), else FR_ERR_TOO_LARGE */
+                              +-1023 (max weighted degree of the graph), and n + nnz below
+                              2^31 - 64, else FR_ERR_TOO_LARGE */
     int32_t mt_alpha;      /* > 0: fr_refine_active runs a multi-try FM pass (Section 4.2) after
                               the pairwise improvements of every matching, its k-way searches
                               stopped by the KaSPar rule p mu^2 > mt_alpha sigma^2 + ln n

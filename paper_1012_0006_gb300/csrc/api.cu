@@ -272,6 +272,10 @@ fr_status ensure_base(fr_ctx *ctx, int n, int nnz, int k, int reps) {
 }
 
 fr_status ensure_fm(fr_ctx *ctx, int n, int nnz, int k, int P) {
+    if (!fm_entries_fit(n, nnz)) {
+        ctx_error(ctx, "FM: n + nnz exceeds the entry index range");
+        return FR_ERR_TOO_LARGE;
+    }
     ctx->fm_live = true;
     if (ctx->fm_mem && n <= ctx->fm_n && nnz <= ctx->fm_nnz && k <= ctx->fm_k && P <= ctx->fm_p) return FR_OK;
     const long long nn = std::max(n, ctx->fm_n), mm = std::max(nnz, ctx->fm_nnz);

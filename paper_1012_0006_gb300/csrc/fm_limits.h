@@ -1,6 +1,8 @@
 // Limits of the two-way FM search, as plain C++ (checked without a device).
 #pragma once
 
+#include <climits>
+
 #ifdef __CUDACC__
 #define FR_HD __host__ __device__
 #else
@@ -20,5 +22,9 @@ FR_HD constexpr int fm_row_end(int j0, int j1, int nnz) {
     const int end = j1 < nnz ? j1 : nnz;
     return end - j0 > kFmMaxDeg ? j0 + kFmMaxDeg : end;
 }
+
+// Stack entries are counted in 32 bits: at most one per vertex and arc of the graph, and a
+// move looks up to 32 entries past the last one.
+FR_HD constexpr bool fm_entries_fit(long long n, long long nnz) { return n + nnz <= INT_MAX - 64; }
 
 }  // namespace fr

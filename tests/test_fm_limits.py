@@ -13,7 +13,7 @@ def _run(tmp_path, body):
     if not cxx:
         pytest.skip("no g++")
     src, exe = tmp_path / "t.cpp", tmp_path / "t"
-    src.write_text('#include "fm_limits.h"\n#include <climits>\n#include <cstdio>\nusing namespace fr;\n'
+    src.write_text('#include "fm_limits.h"\n#include <cstdio>\n#include <initializer_list>\nusing namespace fr;\n'
                    '#define REQUIRE(x) if (!(x)) { std::printf("line %d: %s\\n", __LINE__, #x); return 1; }\n'
                    "int main() {\n" + body + "\nreturn 0; }\n")
     subprocess.run([cxx, "-std=c++17", "-O1", "-fsanitize=undefined", "-fno-sanitize-recover", "-I", CSRC, str(src),
@@ -36,4 +36,22 @@ def test_a_row_of_two_entries_is_no_longer_than_a_row(tmp_path):
             REQUIRE((long long)end - b[0] <= kFmMaxDeg);
             if (&b == &e) REQUIRE(end == e[1]);
         }
+    """)
+
+
+def test_entries_are_counted_in_32_bits(tmp_path):
+    _run(tmp_path, """
+    const long long most = INT_MAX;
+    for (long long n : {1LL, 1000LL, 1LL << 20, most / 2, most}) {
+        // the largest graph that fits: its last entry + 1, and 32 positions past it, are ints
+        const long long nnz = most - 64 - n;
+        if (nnz >= 0) {
+            REQUIRE(fm_entries_fit(n, nnz));
+            const int end = (int)(n + nnz);
+            REQUIRE(end + 32 > end && end + 1 > 0);
+        }
+        REQUIRE(!fm_entries_fit(n, nnz + 1));
+        REQUIRE(!fm_entries_fit(n, most));
+    }
+    REQUIRE(fm_entries_fit(1 << 30, (1 << 30) - 65));
     """)
