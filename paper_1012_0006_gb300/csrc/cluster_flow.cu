@@ -76,7 +76,7 @@ static cudaError_t cluster_setup() {
     cudaFuncAttributes fa;
     e = cudaFuncGetAttributes(&fa, cluster_flow_kernel<512>);
     if (e != cudaSuccess) return e;
-    const int dyn = optin - (int)fa.sharedSizeBytes - 64;
+    const int dyn = (optin < kClusterSmemMax ? optin : kClusterSmemMax) - (int)fa.sharedSizeBytes - 64;
     e = cudaFuncSetAttribute(cluster_flow_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(cluster_flow_kernel<512>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);

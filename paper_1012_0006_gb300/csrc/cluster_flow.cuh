@@ -46,6 +46,18 @@ struct ClusterHdr {
 };
 static_assert(sizeof(ClusterHdr) <= kHdrBytes, "the header leads the dynamic shared memory");
 
+// Bytes of a vertex and of an arc (packed residuals; 4 more otherwise) in a CTA's shared memory,
+// of an arc into another CTA in the remote tables, and the widths of the places of vertices
+// and arcs.  A launch asks for no more shared memory than these widths can address, whatever
+// the device offers (227 KB on sm_103a).
+constexpr int kVtxBytes = 31, kArcBytes = 8, kRemoteBytes = 10;
+constexpr int kVtxBits = 13, kArcBits = 15;
+constexpr int kClusterSmemMax = 227 * 1024;
+static_assert((kClusterSmemMax - kHdrBytes) / kVtxBytes <= 1 << kVtxBits, "a vertex's place");
+static_assert((kClusterSmemMax - kHdrBytes) / kArcBytes <= 1 << kArcBits, "an arc's place");
+static_assert((kClusterSmemMax - kHdrBytes) / kRemoteBytes <= 1 << 16, "a remote slot in 16 bits");
+static_assert(kClusterMax <= 1 << (32 - kVtxBits - kArcBits), "a rank above both places");
+
 // Distributed shared memory by explicit address: a shared::cluster address (32 bits) of an
 // element of some CTA's shared memory, and plain loads / relaxed reductions at it.  Every
 // CTA carves its arrays at the same offsets, so the address of array X at the same index
@@ -118,8 +130,7 @@ struct ClusterFlow {
     __device__ __forceinline__ int cs(int a) const { return narrow ? (int)((unsigned)res[a] >> 16) : csum[a]; }
     __device__ __forceinline__ void set_rs(int a, int v) { res[a] = narrow ? ((res[a] & ~0xFFFF) | v) : v; }
     // Per arc, one word.  An arc whose head this CTA holds: its rank, the head's index and
-    // the index of the reverse arc (a CTA's shared memory holds fewer than 2^13 vertices of
-    // 31 bytes and 2^15 arcs of 8).  An arc into another CTA: another rank, and a slot of the
+    // the index of the reverse arc.  An arc into another CTA: another rank, and a slot of the
     // remote tables, which hold the same three for it (rw), a copy of the head's label (rg)
     // and the slot of the reverse arc in the head's CTA (rslot).  With the residual an arc is
     // 8 bytes, 18 if remote: cluster-wide addresses of both and a copy of every head's label
@@ -134,7 +145,6 @@ struct ClusterFlow {
     ShArr<unsigned char> bord;
     int rot, arot;             // rotating counter and vote indexes (identical in every CTA)
 
-    static constexpr int kVtxBits = 13, kArcBits = 15;
     static __device__ __forceinline__ unsigned pack_adr(int rk, int v, int a) {
         return ((unsigned)rk << (kVtxBits + kArcBits)) | ((unsigned)v << kArcBits) | (unsigned)a;
     }
@@ -333,7 +343,7 @@ struct ClusterFlow {
         csum.o = narrow ? 0u : take(4u * nacap);
         queue.o = take(2 * kQueue * sizeof(int2));
         // the rest: the remote tables
-        nrcap = (int)(smem_bytes - p - 48) / 10;
+        nrcap = (int)(smem_bytes - p - 48) / kRemoteBytes;
         rw.o = take(4u * nrcap);
         rg.o = take(4u * nrcap);
         rslot.o = p;
@@ -346,6 +356,7 @@ struct ClusterFlow {
         o_cla = cla.o - lab.o;
     }
 
+    // (4 bytes a vertex more than carve takes: what is left is room for the remote tables)
     static __host__ __device__ size_t bytes_for(int nvcap, int nacap, bool narrow) {
         auto a = [](size_t b) { return (b + 15) / 16 * 16; };
         return kHdrBytes + 7 * a(4ull * nvcap) + a(4ull * (nvcap + 1)) + a(nvcap) + a(2ull * nvcap) + (narrow ? 2 : 3) * a(4ull * nacap) +
@@ -421,9 +432,9 @@ struct ClusterFlow {
         // for the largest range's vertices and arcs, so the first candidate that fits
         // shared memory is taken: the arc split where it fits, the others where the
         // order of the vertices puts many light vertices together.
-        const int ab = w.narrow ? 8 : 12;
+        const int ab = w.narrow ? kArcBytes : kArcBytes + 4;
         {
-            const long long Btot = 31LL * V + (long long)ab * A;
+            const long long Btot = (long long)kVtxBytes * V + (long long)ab * A;
             const long long tot3[3] = {(long long)A, Btot, (long long)V};
             const int per = (V + C - 1) / C;
             const int k0 = min(V, per * rank), k1 = min(V, k0 + per);
@@ -436,7 +447,7 @@ struct ClusterFlow {
             }
             int tot, btot;
             const int e0 = block_exclusive_scan<TPB>(mine, &tot);
-            const int b0 = block_exclusive_scan<TPB>(31 * (s1 - s0) + ab * mine, &btot);
+            const int b0 = block_exclusive_scan<TPB>(kVtxBytes * (s1 - s0) + ab * mine, &btot);
             if (threadIdx.x == 0) {
                 hdr0->counts[rank] = tot;
                 hdr0->counts2[rank] = btot;
@@ -466,7 +477,7 @@ struct ClusterFlow {
             for (int k = s0; k < s1; ++k) {
                 const int i = __ldcg(&pmem[k]);
                 const int d = w.off[i + 1] - w.off[i];
-                const int b = 31 + ab * d;
+                const int b = kVtxBytes + ab * d;
                 pacs[k] = run;
                 const long long lo3[3] = {(long long)run, brun, (long long)k};
                 const long long sz3[3] = {(long long)d, (long long)b, 1};

@@ -190,7 +190,7 @@ static cudaError_t queue_setup() {
     cudaFuncAttributes fa;
     e = cudaFuncGetAttributes(&fa, queue_kernel<512>);
     if (e != cudaSuccess) return e;
-    const int dyn = optin - (int)fa.sharedSizeBytes - 64;
+    const int dyn = (optin < kClusterSmemMax ? optin : kClusterSmemMax) - (int)fa.sharedSizeBytes - 64;
     e = cudaFuncSetAttribute(queue_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(queue_kernel<512>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
