@@ -781,7 +781,9 @@ static fr_status run_pair_iteration(fr_ctx *ctx, const fr_graph *g, int32_t *par
     // one launch of one cluster where the corridor fits
     const int tq = queue_round_size(ctx, 1, est, (double)g->nnz / g->n, opt);
     if (tq >= 0) {
-        PairDev *hp = reinterpret_cast<PairDev *>(ctx->h_stage + 1024);
+        // (staged beside setup_single's bytes, which are written without a synchronisation when
+        // the workspace is refused)
+        PairDev *hp = reinterpret_cast<PairDev *>(ctx->h_stage + 1600);
         hp->g = 0; hp->a = a; hp->b = b; hp->mb = mb; hp->Ubase = Ubase;
         CK(cudaMemcpyAsync(ctx->pairs, hp, sizeof(PairDev), cudaMemcpyHostToDevice, ctx->stream));
         CK(cudaMemsetAsync(ctx->sides, 0, 2 * sizeof(SideDev), ctx->stream));
