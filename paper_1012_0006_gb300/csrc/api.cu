@@ -673,9 +673,9 @@ cudaError_t launch_clusters(fr_ctx *ctx, Work &w, long long est_pair_vertices, d
                             cudaStream_t st, int *nl) {
     *nl = 0;
     const int T = fr_ctx::kNumClusterSizes;
-    // shared memory a pair needs: ~29 B per vertex and 11 B per arc (15 B when
-    // capacities do not pack into 16 bits), plus a little for an uneven split; a CTA
-    // has cluster_flow_smem() bytes
+    // shared memory a pair needs, estimated: ~29 B per vertex (it takes 31) and 11 B per arc
+    // (8, and 10 more for one into another CTA; 4 more when capacities do not pack into 16
+    // bits), plus a little for an uneven split; a CTA has cluster_flow_smem() bytes
     const double need = 1.05 * (double)est_pair_vertices * (29.0 + (w.narrow ? 11.0 : 15.0) * avg_degree);
     const double per_cta = 0.95 * (double)cluster_flow_smem();
     // Among the sizes that hold the estimate, the one with the least expected time:

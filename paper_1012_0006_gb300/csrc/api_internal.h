@@ -213,7 +213,7 @@ fr::FmDev fm_view(fr_ctx *ctx, int p0, const fr_options *opt);
 // Launches of one flow iteration over the pairs of w after the boundary scan:
 // step (BFS, ids, build) -> cluster max flow -> step (rest), or one step kernel.
 // est_pair_vertices: estimated corridor size of the largest pair (chooses the cluster size);
-// cluster_ctas: 4, 8 or 16 forces the first cluster size, 0 chooses it.
+// cluster_ctas: forces the first cluster size (one of kClusterSizes), 0 chooses it.
 cudaError_t launch_round(fr_ctx *ctx, fr::Work &w, int grid, int tpb, cudaStream_t st, cudaEvent_t *ev,
                          long long est_pair_vertices = 0, double avg_degree = 12.0, int cluster_ctas = 0);
 cudaError_t launch_clusters(fr_ctx *ctx, fr::Work &w, long long est_pair_vertices, double avg_degree, int force,

@@ -50,10 +50,10 @@ struct QCaps {
     long long nu, mu, vq, words, swords;
 };
 
-// Per-pair capacities of a cluster of `ctas` CTAs: a network that fits its shared
-// memory has at most dyn / 29 vertices; arcs have room for dyn / 16 per CTA (8 bytes each
-// would fit, but a pair that large is better off on a larger cluster, and the HBM arrays of
-// every slot would double).
+// Per-pair capacities of a cluster of `ctas` CTAs: dyn / 28 vertices per CTA, more than its
+// shared memory holds (31 bytes a vertex, see ClusterFlow::carve); arcs have room for dyn / 16
+// (8 bytes each would fit, but a pair that large is better off on a larger cluster, and the
+// HBM arrays of every slot would double).
 QCaps caps_for(int ctas, int n) {
     const long long dyn = (long long)queue_smem();
     QCaps c;
@@ -253,7 +253,8 @@ int queue_size_for(fr_ctx *ctx, const BatchPlan &pl, const fr_options *opt) {
     // bound the size is the one with the most pairs in flight over a pair's time, whatever is
     // fastest, so that no call is refused for speed.
     const bool bounded = ctx->arena_limit != 0;
-    // (16 bytes an arc: the arcs a slot has room for, see caps_for)
+    // (an estimate: 31 bytes a vertex rounded down, and 16 an arc, the arcs a slot has room for,
+    // see caps_for)
     const double need = 1.05 * (double)est * (29.0 + (bounded && !ctx->narrow_ok ? 20.0 : 16.0) * pl.avg_degree);
     const double per_cta = 0.95 * (double)dyn;
     const int force = opt->cluster_ctas ? opt->cluster_ctas : ctx->tune_ctas;
@@ -480,7 +481,7 @@ fr_status run_queue_sweep(fr_ctx *ctx, const fr_graph *g, int32_t *part, const B
 
 int queue_round_size(fr_ctx *ctx, int P, long long est, double avg_degree, const fr_options *opt) {
     if (P <= 0 || opt->sweep_sched == 1 || ctx->max_clusters <= 0 || queue_smem() == 0) return -1;
-    const double need = 1.05 * (double)est * (29.0 + 16.0 * avg_degree);
+    const double need = 1.05 * (double)est * (29.0 + 16.0 * avg_degree);   // (as for a sweep)
     const double per_cta = 0.95 * (double)queue_smem();
     const int force = opt->cluster_ctas ? opt->cluster_ctas : ctx->tune_ctas;
     int best = -1, kept = -1;

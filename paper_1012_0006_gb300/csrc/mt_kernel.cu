@@ -28,8 +28,8 @@
 // follow from their records alone: a move is the popped entry, x's arcs, the neighbours'
 // records.  Summing every neighbour's arcs again instead, as first built, read two more
 // dependent levels (arcs, their blocks) for every neighbour: the global rounds of a 3D
-// rgg of 524,288 vertices and 64 blocks (29,191 moves) took 90 ms so and take 50.5 ms now,
-// about 3,400 cycles a move, half of it loads that miss L1 (300 cycles near in L2, some 700
+// rgg of 524,288 vertices and 64 blocks (29,191 moves) took 90 ms so and take 48.7 ms now,
+// about 3,300 cycles a move, half of it loads that miss L1 (300 cycles near in L2, some 700
 // when first touched) and half the warp's own instructions.  The queue is an array of gain buckets, each a stack of 16-byte entries in global memory with
 // its top and a non-empty bitmap in shared memory; an entry carries what the move needs
 // (vertex, target, block, adjacency range) and is live while that word is not zero: keying
