@@ -786,8 +786,6 @@ static fr_status run_pair_iteration(fr_ctx *ctx, const fr_graph *g, int32_t *par
         PairDev *hp = reinterpret_cast<PairDev *>(ctx->h_stage + 1600);
         hp->g = 0; hp->a = a; hp->b = b; hp->mb = mb; hp->Ubase = Ubase;
         CK(cudaMemcpyAsync(ctx->pairs, hp, sizeof(PairDev), cudaMemcpyHostToDevice, ctx->stream));
-        CK(cudaMemsetAsync(ctx->sides, 0, 2 * sizeof(SideDev), ctx->stream));
-        CK(cudaMemsetAsync(ctx->pacc, 0, sizeof(PairAcc), ctx->stream));
         RoundQueue rq;
         fr_status sq = enqueue_round_queue(ctx, g, part, k, 1, Lmax, opt, tq, &rq);
         if (sq != FR_OK) return sq;

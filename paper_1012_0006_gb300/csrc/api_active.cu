@@ -75,12 +75,17 @@ fr_status run_pairs_step(fr_ctx *ctx, const fr_graph *g, int32_t *part, int32_t 
         hs[ps[i].a] = 2 * i;
         hs[ps[i].b] = 2 * i + 1;
     }
-    CK(cudaMemcpyAsync(ctx->graphs, h, sizeof(gd), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(ctx->pairs, hp, sizeof(PairDev) * P, cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaMemcpyAsync(ctx->sob1, hs, sizeof(int) * k, cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaMemsetAsync(ctx->ctl, 0, sizeof(Ctl), ctx->stream));
-    CK(cudaMemsetAsync(ctx->sides, 0, sizeof(SideDev) * 2 * P, ctx->stream));
-    CK(cudaMemsetAsync(ctx->pacc, 0, sizeof(PairAcc) * P, ctx->stream));
+    // what only the FM step and the round's own launches read
+    bool described = false;
+    auto describe = [&]() -> fr_status {
+        if (described) return FR_OK;
+        CK(cudaMemcpyAsync(ctx->graphs, h, sizeof(gd), cudaMemcpyHostToDevice, ctx->stream));
+        CK(cudaMemcpyAsync(ctx->sob1, hs, sizeof(int) * k, cudaMemcpyHostToDevice, ctx->stream));
+        CK(cudaMemsetAsync(ctx->ctl, 0, sizeof(Ctl), ctx->stream));
+        described = true;
+        return FR_OK;
+    };
     Work w = make_work(ctx, 0, 0, P, g->n, opt);
     const int tpb = choose_tpb(ctx, opt);
     const double avgc = std::max(1.0, (double)W / g->n);
@@ -93,6 +98,7 @@ fr_status run_pairs_step(fr_ctx *ctx, const fr_graph *g, int32_t *part, int32_t 
     const int grid = choose_grid(ctx, opt, tpb, 2 * P, std::max(1LL, est));
     if (fm_first) {
         int nf = 0;
+        if ((st = describe()) != FR_OK) return st;
         CK(launch_fm(w, fm_view(ctx, 0, opt), k, ctx->sms, ctx->stream, &nf));
     }
     // one launch of clusters where the corridors fit, else the round's own sequence
@@ -100,6 +106,10 @@ fr_status run_pairs_step(fr_ctx *ctx, const fr_graph *g, int32_t *part, int32_t 
     const int tq = queue_round_size(ctx, P, emax, (double)g->nnz / g->n, opt);
     if (tq >= 0 && (st = enqueue_round_queue(ctx, g, part, k, P, Lmax, opt, tq, &rq)) != FR_OK) return st;
     auto own_launches = [&]() -> fr_status {
+        const fr_status ds = describe();
+        if (ds != FR_OK) return ds;
+        CK(cudaMemsetAsync(ctx->sides, 0, sizeof(SideDev) * 2 * P, ctx->stream));
+        CK(cudaMemsetAsync(ctx->pacc, 0, sizeof(PairAcc) * P, ctx->stream));
         CK(cudaMemsetAsync(ctx->hist, 0, sizeof(long long) * 3 * 2 * (size_t)P * kHistBins, ctx->stream));
         CK(launch_scan_list(w, 0, ctx->stream));
         CK(launch_round(ctx, w, grid, tpb, ctx->stream, nullptr, emax, (double)g->nnz / g->n,
@@ -119,7 +129,8 @@ fr_status run_pairs_step(fr_ctx *ctx, const fr_graph *g, int32_t *part, int32_t 
     auto read_back = [&]() -> fr_status {
         CK(cudaMemcpyAsync(ha, ctx->pacc, sizeof(PairAcc) * P, cudaMemcpyDeviceToHost, ctx->stream));
         CK(cudaMemcpyAsync(hsd, ctx->sides, sizeof(SideDev) * 2 * P, cudaMemcpyDeviceToHost, ctx->stream));
-        CK(cudaMemcpyAsync(hc, ctx->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, ctx->stream));
+        if (described) CK(cudaMemcpyAsync(hc, ctx->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, ctx->stream));
+        else memset(hc, 0, sizeof(Ctl));
         CK(cudaStreamSynchronize(ctx->stream));
         return FR_OK;
     };
@@ -130,8 +141,6 @@ fr_status run_pairs_step(fr_ctx *ctx, const fr_graph *g, int32_t *part, int32_t 
         qst = finish_round_queue(ctx, g, part, k, "fr_refine_active", &rq);
         if (qst == FR_OK && !rq.queued && hc->error == 0) {   // a pair outgrew its cluster
             queued = false;
-            CK(cudaMemsetAsync(ctx->sides, 0, sizeof(SideDev) * 2 * P, ctx->stream));
-            CK(cudaMemsetAsync(ctx->pacc, 0, sizeof(PairAcc) * P, ctx->stream));
             if ((st = own_launches()) != FR_OK || (st = read_back()) != FR_OK) return st;
         }
     }

@@ -42,6 +42,7 @@ struct QueueMem {
     int *qb_sorted = nullptr, *qb_start = nullptr, *qb_cnt = nullptr, *qb_app = nullptr, *qb_pool = nullptr,
         *qb_lst = nullptr;
     int qb_cap = 0;
+    long long *blockw0 = nullptr;              // rounds only: [k] the block weights before the launch
 };
 
 struct fr_ctx {
@@ -231,7 +232,7 @@ int queue_size_for(fr_ctx *ctx, const BatchPlan &pl, const fr_options *opt);
 fr_status run_queue_sweep(fr_ctx *ctx, const fr_graph *g, int32_t *part, const BatchPlan &pl, const fr_options *opt,
                           int t, float *ms, bool *ran, std::vector<fr::Ctl> *ctls);
 // One round of block-disjoint pairs as one launch of the queue kernel, each pair in a
-// cluster (ctx->pairs uploaded, ctx->sides and ctx->pacc cleared by the caller).
+// cluster (ctx->pairs uploaded by the caller; ctx->sides and ctx->pacc are cleared).
 // queue_round_size: index into kClusterSizes for P pairs whose largest corridor is estimated
 // at est vertices, or -1 where it does not apply.  enqueue: rq->queued = false if the arena
 // bound leaves no room.  After the caller synchronised the stream, finish reads what the

@@ -39,9 +39,8 @@ constexpr double kRelTiny[fr_ctx::kNumClusterSizes] = {1.0, 1.01, 1.02, 1.06, 1.
 // host staging offsets (the first megabytes of h_stage belong to the other paths)
 constexpr size_t kStageGraphs = 4u << 20;
 constexpr size_t kStagePrev = (4u << 20) + (64u << 10);
-// a round on the queue kernel (run_round_queue): descriptors, block weights, read-back
-constexpr size_t kStageRound = 6u << 20, kStageRoundW = (6u << 20) + (256u << 10),
-                 kStageRoundCtl = (6u << 20) + (512u << 10);
+// a round on the queue kernel (enqueue_round_queue): descriptors, read-back
+constexpr size_t kStageRound = 6u << 20, kStageRoundCtl = (6u << 20) + (512u << 10);
 constexpr unsigned long long kWaitNs = 10ull * 1000 * 1000 * 1000;   // one dependency wait, at most 10 s
 
 size_t al256(size_t b) { return (b + 255) / 256 * 256; }
@@ -111,6 +110,7 @@ size_t queue_bytes(int ctas, int clusters, int n, int nnz, int k, int reps, int 
     size_t b = 2 * al256(4) + al256(4ull * nnz) + al256(sizeof(QSlot) * clusters) + al256(sizeof(GraphDev) * clusters) +
                al256(sizeof(QueueMem::QCtl) * clusters) + al256(32ull * clusters) +
                slot_bytes(caps_for(ctas, n), ctas, k, reps) * clusters;
+    if (!lists) b += al256(8ull * k);   // blockw0
     if (lists)
         b += al256(8ull * np) + 2 * al256(4ull * n) + al256(4ull * (k + 1)) + 2 * al256(4ull * k) +
              al256(4ull * k * qb_cap_for(n, k));
@@ -177,6 +177,8 @@ fr_status ensure_queue(fr_ctx *ctx, QueueMem &Q, int ctas, int clusters, int n, 
         Q.qb_cap = (int)qb_cap_for(nn, kk);
         Q.qb_pool = take<int>(p, (long long)kk * Q.qb_cap);
         Q.qb_lst = take<int>(p, nn);
+    } else {
+        Q.blockw0 = take<long long>(p, kk);
     }
     Q.graphs = take<GraphDev>(p, cc);
     Q.host.assign(cc, QSlot());
@@ -518,7 +520,7 @@ fr_status enqueue_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int
     if (st == FR_ERR_OOM) return FR_OK;   // no room under the arena bound: the round's own launches
     if (st != FR_OK) return st;
     GraphDev *hg = reinterpret_cast<GraphDev *>(ctx->h_stage + kStageRound);
-    static_assert(kStageRound + 64 * sizeof(GraphDev) <= kStageRoundW, "descriptors of every resident cluster");
+    static_assert(kStageRound + 64 * sizeof(GraphDev) <= kStageRoundCtl, "descriptors of every resident cluster");
     if (clusters > 64) clusters = 64;
     for (int i = 0; i < clusters; ++i) {
         GraphDev &gd = hg[i];
@@ -531,10 +533,6 @@ fr_status enqueue_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int
         gd.bl = ctx->bl; gd.blc = ctx->blc; gd.inb = ctx->inb;
     }
     CK(cudaMemcpyAsync(Q.graphs, hg, sizeof(GraphDev) * (size_t)clusters, cudaMemcpyHostToDevice, ctx->stream));
-    // part and the block weights as they are, should a pair outgrow its cluster
-    CK(cudaMemcpyAsync(ctx->spare, part, sizeof(int) * (size_t)g->n, cudaMemcpyDeviceToDevice, ctx->stream));
-    CK(cudaMemcpyAsync(ctx->h_stage + kStageRoundW, ctx->blockw, sizeof(long long) * (size_t)k, cudaMemcpyDeviceToHost,
-                       ctx->stream));
     QueueArgs q;
     memset(&q, 0, sizeof(q));
     q.wt = make_work(ctx, 0, 0, P, g->n, opt);
@@ -549,11 +547,15 @@ fr_status enqueue_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int
     q.prev = nullptr;   // no pair waits for another
     q.gabort = Q.gabort;
     q.wait_ns = kWaitNs;
-    CK(cudaMemsetAsync(Q.ticket, 0, queue_state_bytes(Q, clusters), ctx->stream));
-    if (P > 1) {   // pairs commit to the list while others scan it: they scan what is on it now
-        q.wt.scan_len = Q.ticket + 2;
-        CK(cudaMemcpyAsync(Q.ticket + 2, ctx->blc, sizeof(int), cudaMemcpyDeviceToDevice, ctx->stream));
-    }
+    q.wt.scan_len = Q.ticket + 2;   // pairs commit to the list while others scan it: they scan what is on it now
+    RoundBegin rb;
+    rb.part = part; rb.part0 = ctx->spare; rb.n = g->n;
+    rb.blockw = ctx->blockw; rb.blockw0 = Q.blockw0; rb.k = k;
+    rb.clear[0] = reinterpret_cast<int *>(ctx->sides); rb.words[0] = (int)(sizeof(SideDev) / 4 * 2 * (size_t)P);
+    rb.clear[1] = reinterpret_cast<int *>(ctx->pacc); rb.words[1] = (int)(sizeof(PairAcc) / 4 * (size_t)P);
+    rb.clear[2] = Q.ticket; rb.words[2] = (int)(queue_state_bytes(Q, clusters) / 4);
+    rb.blc = ctx->blc; rb.scan_len = Q.ticket + 2;
+    CK(launch_round_begin(rb, ctx->sms, ctx->stream));
     CK(launch_queue_sweep(q, ctas, clusters, ctx->stream));
     char *h = ctx->h_stage + kStageRoundCtl;
     CK(cudaMemcpyAsync(h, Q.gabort, 256 + sizeof(QueueMem::QCtl) * (size_t)clusters, cudaMemcpyDeviceToHost,
@@ -586,8 +588,8 @@ fr_status finish_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int 
         rq->queued = false;
         ++ctx->queue_fallbacks;
         CK(cudaMemcpyAsync(part, ctx->spare, sizeof(int) * (size_t)g->n, cudaMemcpyDeviceToDevice, ctx->stream));
-        CK(cudaMemcpyAsync(ctx->blockw, ctx->h_stage + kStageRoundW, sizeof(long long) * (size_t)k,
-                           cudaMemcpyHostToDevice, ctx->stream));
+        CK(cudaMemcpyAsync(ctx->blockw, ctx->round_q.blockw0, sizeof(long long) * (size_t)k, cudaMemcpyDeviceToDevice,
+                           ctx->stream));
         return FR_OK;
     }
     if (!rq->ctl.error) rq->ctl.error = gab;

@@ -189,7 +189,7 @@ struct Work {
     int gap_interval;            // pulses between gap checks of push-relabel (0: none)
     int *wave_votes;             // queue sweep: this pair starts with a wave, and tells whether it paid (NULL: not)
     const int *scan_len;         // round on the queue kernel: length of the candidate list when the round began
-                                 // (NULL: no other pair's commit runs beside the scan, *blc holds it)
+                                 // (NULL: no commit runs beside the scan, *blc holds it)
     unsigned long long seed;
     long long pulse_cap;
     int *crank;                  // per graph arc: rank among its row's corridor arcs (NULL: outs holds it)

@@ -19,6 +19,7 @@
 // stops the sweep with E_MISFIT, and the host runs it again round by round.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <climits>
 
 #include "cluster_flow.cuh"
@@ -174,6 +175,28 @@ __global__ void __launch_bounds__(TPB, 1) queue_kernel(QueueArgs q, size_t smem_
         }
     }
     cl.sync();   // no CTA exits while another may still read its shared memory
+}
+
+__global__ void __launch_bounds__(256) round_begin_kernel(RoundBegin r) {
+    const int t = blockIdx.x * 256 + threadIdx.x, nt = gridDim.x * 256;
+    for (long long i = t; i < r.n; i += 4LL * nt) {
+        int v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = i + (long long)u * nt < r.n ? r.part[i + (long long)u * nt] : 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i + (long long)u * nt < r.n) r.part0[i + (long long)u * nt] = v[u];
+    }
+    for (int i = t; i < r.k; i += nt) r.blockw0[i] = r.blockw[i];
+    for (int a = 0; a < 3; ++a)
+        for (int i = t; i < r.words[a]; i += nt) r.clear[a][i] = r.clear[a] + i == r.scan_len ? *r.blc : 0;
+}
+
+cudaError_t launch_round_begin(const RoundBegin &r, int sms, cudaStream_t st) {
+    const int most = std::max({r.n / 4, r.k, r.words[0], r.words[1], r.words[2]});
+    const int grid = std::max(1, std::min((most + 255) / 256, 4 * sms));
+    round_begin_kernel<<<grid, 256, 0, st>>>(r);
+    return cudaGetLastError();
 }
 
 // Dynamic shared memory of the queue kernel: the opt-in maximum per block minus its

@@ -46,6 +46,25 @@ struct QueueArgs {
     unsigned long long wait_ns;   // bound of one wait for a dependency (then E_ABORT)
 };
 
+// What a single round does before its launch, in one kernel instead of six copies and clears
+// of 1.5-2 us each: part and the block weights kept, should a pair outgrow its cluster, the
+// pairs' and the launch's state cleared, the length of the candidate list taken.  Bound by
+// that fixed cost up to about a million vertices, by the copy of part above.  Together with
+// uploads that only the FM step and the round's own launches need: the pair of the 64 x 64
+// grid 270 -> 253 us, two outer rounds of active scheduling on rgg3d 4,096 vertices, k = 8,
+// 2.88 -> 2.45 ms (2.65 with the round's own launches), on 30,011, k = 32, 8.41 -> 7.22.
+struct RoundBegin {
+    const int *part;
+    int *part0;                // [n]
+    const long long *blockw;
+    long long *blockw0;        // [k]
+    int n, k;
+    int *clear[3];             // cleared: words[i] words each
+    int words[3];
+    const int *blc;
+    int *scan_len;             // a word of clear[2]: set to *blc
+};
+cudaError_t launch_round_begin(const RoundBegin &r, int sms, cudaStream_t st);
 cudaError_t launch_queue_sweep(const QueueArgs &q, int cluster, int clusters, cudaStream_t st);
 // Clusters of `cluster` CTAs the queue kernel can keep resident at once (0: none).
 cudaError_t queue_capacity(int cluster, int *max_clusters);
