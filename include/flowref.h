@@ -80,9 +80,10 @@ typedef struct fr_options {
     int32_t inner_ops;     /* push/relabel operations per vertex per pulse; 0 = default */
     int32_t pulse_passes;  /* lock-free pulse passes between grid barriers; 0 = default */
     int32_t flow_sched;    /* per-pair cluster max flow: 1 level-ordered waves, 2 lock-free pulses;
-                              0 = tuned default (pulses unless fr_autotune chose waves; in a queue
-                              sweep some pairs try a wave, and pairs go on in waves where it pays).
-                              Results do not depend on it */
+                              0 = tuned default (pulses unless fr_autotune chose waves or the graph's
+                              weighted degrees are at most 4; in a queue sweep some pairs try a wave,
+                              with weighted degrees of at most 6 every pair of a round does, and
+                              pairs go on in waves where it pays).  Results do not depend on it */
     int32_t cluster_ctas;  /* CTAs of the first per-pair cluster launch (4, 6, 8, 12 or 16); 0 = by the
                               estimated corridor size.  Pairs that do not fit go to 16-CTA
                               clusters, then to the grid-wide flow; results do not depend on it */

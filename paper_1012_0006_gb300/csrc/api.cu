@@ -398,6 +398,9 @@ Work make_work(fr_ctx *ctx, int r, int p0, int P, int n, const fr_options *opt) 
     w.inner = opt && opt->inner_ops > 0 ? opt->inner_ops : ctx->tune_inner;
     w.passes = opt && opt->pulse_passes > 0 ? opt->pulse_passes : ctx->tune_passes;
     w.flow_sched = opt && opt->flow_sched ? opt->flow_sched : ctx->tune_sched;
+    if (w.flow_sched == 0 && low_degree(ctx, kWaveDeg)) w.flow_sched = 1;
+    // (a round's own launches: every pair starts with a wave; the votes are not read)
+    w.wave_votes = w.flow_sched == 0 && low_degree(ctx, kTryDeg) ? ctx->flags : nullptr;
     w.any_mb = opt && opt->mb ? 1 : 0;
     w.seed = opt ? opt->seed : 0;
     w.pulse_cap = opt && opt->pulse_cap > 0 ? opt->pulse_cap : (1LL << 20);
@@ -614,6 +617,7 @@ fr_status run_prep(fr_ctx *ctx, const fr_graph *g, const int32_t *part, int32_t 
     CK(cudaMemcpyAsync(h, ctx->prep, sizeof(PrepOut), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     *host_out = *h;
+    ctx->max_wdeg = h->maxwdeg;
     ctx->narrow_ok = h->maxw < (1 << 15) ? 1 : 0;
     if (h->err) {
         ctx_error(ctx, h->err == E_TOO_LARGE ? "weighted degree >= 2^30" :

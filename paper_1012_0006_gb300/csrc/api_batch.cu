@@ -406,7 +406,7 @@ static fr_status run_sweep(fr_ctx *ctx, const fr_graph *g, int32_t *part, const 
                                   opt->pulse_passes, ctx->tune_passes, (long long)(uintptr_t)ctx->reps_mem,
                                   opt->flow_sched, opt->cluster_ctas, ctx->tune_ctas, ctx->tune_sched,
                                   ctx->narrow_ok, opt->pre_waves, ctx->tune_prewaves, opt->fm_permille,
-                                  opt->gap_interval,
+                                  opt->gap_interval, low_degree(ctx, kWaveDeg), low_degree(ctx, kTryDeg),
                                   (long long)(uintptr_t)ctx->fm_mem};
     for (int r = 0; r <= pl.nr; ++r) key.push_back(pl.off[r]);
     for (int r = 0; r < pl.nr; ++r) key.push_back(pl.grid[r]);

@@ -59,6 +59,7 @@ struct fr_ctx {
     int tune_ctas = 0;   // first cluster size (0: by the estimated corridor size)
     int tune_sched = 0;  // cluster max-flow schedule (fr_options.flow_sched)
     int tune_prewaves = 0;   // waves before the first pulse (fr_options.pre_waves)
+    int max_wdeg = 0;    // weighted degree of the last prep's graph, at most (0: no prep yet)
     int narrow_ok = 0;   // the last prep found every edge weight < 2^15 (packed residuals in clusters)
     // per-pair max flow in thread-block clusters of kClusterSizes[t] CTAs: how many of
     // each can be resident (all 0: grid-wide path only); max_clusters = the largest
@@ -90,7 +91,7 @@ struct fr_ctx {
     unsigned int *qbits = nullptr, *used = nullptr;
     int *sob_round = nullptr, *pair_a = nullptr, *pair_b = nullptr, *pair_round = nullptr, *round_off = nullptr;
     fr::PrepOut *prep = nullptr;
-    int *sob1 = nullptr, *flags = nullptr;
+    int *sob1 = nullptr, *flags = nullptr;   // flags: [0] votes of rounds whose pairs start with a wave (make_work)
     // pair-count workspace
     void *pair_mem = nullptr;
     size_t pair_bytes = 0;
@@ -184,6 +185,18 @@ fr_status ensure_pairs(fr_ctx *ctx, int P, int R, int reps);
 fr_status ensure_reps(fr_ctx *ctx, int reps);
 fr::Work make_work(fr_ctx *ctx, int r, int p0, int P, int n, const fr_options *opt);
 int choose_tpb(fr_ctx *ctx, const fr_options *opt);
+// Graphs of few arcs a vertex (their weighted degrees bounded by most; known after a prep).  A
+// scan or a pass of the pulses costs two block barriers however little there is to do, and the
+// networks of such graphs have long distances: since the passes work on lists, pulses take
+// longer on them.  With weighted degrees up to kWaveDeg the flows run in waves (2D grid 256 x
+// 256, k = 16, alpha 4: a sweep 7.3 ms before the lists, 8.2 with them, 6.4 in waves, a pair 0.99,
+// 1.20, 0.79; ladders, hexagons, grids with edges missing: 0 to 80 % less time).  Up to kTryDeg
+// every pair of a round starts with a wave and goes on in waves where it pays (3D grid of
+// 64^3, k = 8, alpha 4: a pair 1.59, 1.88, 1.14 ms, round by round 5.1, 5.9, 3.85; a triangular
+// lattice, where it does not pay: a pair 3.8, 4.2, 4.3).  Above (rggs), a wave leaves two
+// thirds of the excess, and waves take up to twice the time of pulses.
+constexpr int kWaveDeg = 4, kTryDeg = 6;
+inline bool low_degree(const fr_ctx *ctx, int most) { return ctx->max_wdeg > 0 && ctx->max_wdeg <= most; }
 // Pulses between gap checks of push-relabel (fr_options.gap_interval: 0 -> 8, -1 -> none).
 int gap_interval_of(const fr_options *opt);
 int choose_grid(fr_ctx *ctx, const fr_options *opt, int tpb, int nsides, long long est_vertices);

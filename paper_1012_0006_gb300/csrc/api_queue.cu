@@ -369,7 +369,7 @@ fr_status run_queue_sweep(fr_ctx *ctx, const fr_graph *g, int32_t *part, const B
                                   opt->inner_ops, opt->pulse_cap, (long long)(uintptr_t)ctx->base_mem,
                                   (long long)(uintptr_t)ctx->pair_mem, (long long)(uintptr_t)Q.mem,
                                   ctx->tune_gr, ctx->tune_inner, opt->pulse_passes, ctx->tune_passes,
-                                  opt->flow_sched, ctx->tune_sched, ctx->narrow_ok, opt->pre_waves,
+                                  q.wt.flow_sched, ctx->tune_sched, ctx->narrow_ok, opt->pre_waves,
                                   ctx->tune_prewaves, ctas, clusters, pl.Lmax, opt->gap_interval};
     ctx->prof.scan_ms = ctx->prof.step_ms = ctx->prof.cluster_ms = 0;
     ctx->round_ms.clear();
@@ -544,6 +544,7 @@ fr_status enqueue_round_queue(fr_ctx *ctx, const fr_graph *g, int32_t *part, int
     q.slots = Q.slots;
     q.np = P;
     q.ticket = Q.ticket;
+    q.votes = q.wt.flow_sched == 0 && low_degree(ctx, kTryDeg) ? Q.ticket + 1 : nullptr;
     q.prev = nullptr;   // no pair waits for another
     q.gabort = Q.gabort;
     q.wait_ns = kWaitNs;

@@ -92,8 +92,9 @@ __global__ void __launch_bounds__(TPB, 1) queue_kernel(QueueArgs q, size_t smem_
                 }
             }
             s_grab[it & 1] = j;
-            // every eighth pair tries the wave, and any while it has paid more often than not
-            s_try[it & 1] = q.votes && ((j & 7) == 0 || *(volatile int *)q.votes > 0);
+            // every eighth pair of a sweep tries the wave, and any while it has paid more often
+            // than not; a single round's pairs run at once, and all try it
+            s_try[it & 1] = q.votes && (!q.prev || (j & 7) == 0 || *(volatile int *)q.votes > 0);
         }
         cl.sync();
         const int j = *(volatile int *)cl.map_shared_rank(&s_grab[it & 1], 0);
